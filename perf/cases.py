@@ -121,7 +121,7 @@ def _scene(c, seed):
     g = torch.Generator(device="cuda")
     g.manual_seed(seed * 7919 + N)
     rand = lambda *s: torch.rand(*s, generator=g, device="cuda")  # noqa: E731
-    X = torch.tensor(_design(N, 3)[:, 2:], dtype=torch.float32)
+    X = torch.tensor(_design(N, 3)[:, 2:], dtype=torch.float32, device="cuda")
     coef = rand(6, m).mul_(0.3)
     step = rand(m).mul_(0.4).add_(-0.5)
     at = (n_hist + rand(m) * (N - n_hist)).to(torch.int32)
@@ -130,13 +130,13 @@ def _scene(c, seed):
     cloud = rand(m) < miss
     f32 = c["dtype"] == "f32"
     Y = torch.empty((N, m), dtype=torch.float32 if f32 else torch.int16, device="cuda")
-    y, noise, u = torch.empty(m, device="cuda"), torch.empty(m, device="cuda"), torch.empty(m, device="cuda")
+    noise, u = torch.empty(m, device="cuda"), torch.empty(m, device="cuda")
     bits = None
     if c.get("mask"):
         words = torch.randint(-2 ** 31, 2 ** 31, (2, N, (m + 31) // 32), generator=g, device="cuda", dtype=torch.int64)
         bits = (words[0] | words[1]).to(torch.int32)  # three in four dates usable
     for t in range(N):
-        torch.matmul(X[t].cuda(), coef, out=y)
+        y = X[t] @ coef
         noise.normal_(generator=g)
         y.add_(noise, alpha=0.04).add_(0.5)
         y += step * (at <= t)
