@@ -2,7 +2,7 @@
 //
 // The paper obtains lambda "by simulation" of the limiting MOSUM process
 // (Section 2.3; the one printed value, 2.39, is for alpha = 0.05, h/n = 0.5,
-// N/n = 2 in Section 4.3).  Here every thread simulates one path: a Brownian
+// N/n = 2 in Section 4.3).  Here every warp simulates one path: a Brownian
 // motion W on a grid of G steps per unit time up to T = N/n, Gaussian
 // increments of variance 1/G, and the statistic
 //     sup_{t in [1, T]} |W(t) - W(t - h) - h W(1)| / sqrt(log+ t)
@@ -12,61 +12,164 @@
 // Random numbers: per path a SplitMix64 stream (Steele, Lea and Flood, 2014)
 // started from (seed, path), two 53-bit uniforms per normal, Box-Muller
 // (sqrt(-2 ln u1) cos(2 pi u2), u1 in (0, 1]).  The stream advances by a
-// fixed increment per draw, so the lagged value W(t - h) is rebuilt by a
-// second cursor over the same stream instead of being stored.  FP64
-// throughout (the work is small: one thread per path).
+// fixed increment per draw, so any step's normal can be drawn on its own.
+//
+// What bounds it: the normals.  In FP64 (one thread per path, the lagged
+// W(t - h) rebuilt by a second pass over the stream) 1e5 paths of 1816 steps
+// took 52.6 ms, nearly all of it FP64 issue.  Here the normals come from
+// lambda_fixed.cuh (integer arithmetic) and W is a 64-bit fixed-point word, whose
+// step 2^-frac is finer than the rounding of an FP64 W: against 113-bit arithmetic,
+// over 150 such paths, the statistic is off by 1.1e-16 on average and 4.2e-16 at
+// most; in FP64 by 6.6e-16 and 4.8e-15.  Fixed-point sums do not
+// depend on their order, so a warp takes one path, 32 steps at a time: every lane
+// draws one step, a prefix sum over the warp gives W, and the last h G of them
+// stay in a shared-memory ring for W(t - h): 4.3 ms.
 #include <algorithm>
 #include <cmath>
+#include <mutex>
 #include <vector>
 
 #include "bfm_internal.cuh"
+#include "lambda_fixed.cuh"
 
 namespace bfm {
 namespace {
 
 constexpr uint64_t kGolden = 0x9E3779B97F4A7C15ull;  // SplitMix64 increment
+constexpr int kWarps = 4;                             // paths at a time per block
+constexpr double kE = 2.718281828459045235360287;
+constexpr size_t kMaxRingBytes = 200 * 1024;          // rings of a block
 
-__device__ __forceinline__ uint64_t splitmix_next(uint64_t& state) {
-    uint64_t z = (state += kGolden);
+struct LambdaParams {
+    int G, nsteps, ih, reps;
+    int ie;                // last step with log+ (i / G) = 1
+    int ring;              // ring slots per warp (a multiple of 32, >= ih + 32), 0: no ring
+    int frac;              // fraction bits of W
+    uint64_t seed, sd, h;  // sd, h: 1/sqrt(G) and h times 2^64 (h = 1 as 0)
+    double* stats;
+};
+
+__device__ __forceinline__ uint64_t splitmix_mix(uint64_t z) {
     z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
     z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
     return z ^ (z >> 31);
 }
 
-__device__ __forceinline__ double box_muller(uint64_t& state) {
-    const double two_pow_m53 = 1.0 / 9007199254740992.0;
-    const double u1 = ((double)(splitmix_next(state) >> 11) + 1.0) * two_pow_m53;
-    const double u2 = (double)(splitmix_next(state) >> 11) * two_pow_m53;
-    return sqrt(-2.0 * log(u1)) * cos(6.283185307179586476925286766559 * u2);
+// The increment of W (2^-frac steps) whose two draws follow the stream state s.
+__device__ __forceinline__ int64_t increment(uint64_t s, const LambdaParams& P, const uint64_t* ln, const uint32_t* rec) {
+    const uint64_t n = (splitmix_mix(s + kGolden) >> 11) + 1, f = splitmix_mix(s + 2 * kGolden) >> 11;
+    bool neg;
+    const uint64_t z = fixedpt::normal_q58(n, f, ln, rec, neg);     // |z| <= 8.6
+    const uint64_t q = fixedpt::mulhi(z << 2, P.sd);                // 2^60 |z| / sqrt(G)
+    const int sh = 60 - P.frac;
+    const int64_t d = (int64_t)((q + (1ull << (sh - 1))) >> sh);
+    return neg ? -d : d;
 }
 
-// log+(x): 1 for x <= e, log x above (Eq. 4)
-__device__ __forceinline__ double log_plus(double x) {
-    return x <= 2.718281828459045235360287 ? 1.0 : log(x);
-}
-
-__global__ void lambda_paths(double h, int G, int nsteps, int ih, int reps, uint64_t seed, double* stats) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= reps) return;
-    // stream of path r (one discarded draw after seeding)
-    uint64_t s0 = seed * 0xA0761D6478BD642Full + (uint64_t)r * 0xE7037ED1A0B428DBull + 1ull;
-    splitmix_next(s0);
-    const double sd = 1.0 / sqrt((double)G);
-    uint64_t lead = s0, lag = s0;
-    double W = 0.0, Wlag = 0.0;
-    for (int i = 1; i <= G; ++i) W += sd * box_muller(lead);  // W(1)
-    const double w1 = W;
-    for (int j = 1; j <= G - ih; ++j) Wlag += sd * box_muller(lag);  // W(1 - h)
-    double best = 0.0;
-    for (int i = G;; ++i) {
-        const double z = W - Wlag - h * w1;
-        const double v = fabs(z) / sqrt(log_plus((double)i / (double)G));
-        best = v > best ? v : best;
-        if (i == nsteps) break;
-        W += sd * box_muller(lead);
-        Wlag += sd * box_muller(lag);
+__device__ __forceinline__ int64_t warp_scan(int64_t v, int lane) {  // inclusive sums over the lanes
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int64_t t = __shfl_up_sync(~0u, v, o);
+        v += lane >= o ? t : 0;
     }
-    stats[r] = best;
+    return v;
+}
+
+// One path per warp.  kRing: W(t - h) from the ring; otherwise (h G too long for
+// shared memory) rebuilt from the stream by a second draw of the lagged steps.
+template <bool kRing>
+__global__ void __launch_bounds__(32 * kWarps)
+    lambda_paths(const __grid_constant__ fixedpt::LogTable tab, const LambdaParams P) {
+    __shared__ uint64_t s_ln[256];
+    __shared__ uint32_t s_rec[256];
+    extern __shared__ int64_t s_ring[];
+    for (int i = threadIdx.x; i < 256; i += 32 * kWarps) {
+        s_ln[i] = tab.ln[i];
+        s_rec[i] = fixedpt::log_recip((uint32_t)i);
+    }
+    __syncthreads();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int64_t* ring = s_ring + warp * P.ring;
+    const double unit = ldexp(1.0, -P.frac);
+    for (int64_t r = (int64_t)blockIdx.x * kWarps + warp; r < P.reps; r += (int64_t)gridDim.x * kWarps) {
+        // stream of path r (one discarded draw after seeding); step i uses draws 2i - 1 and 2i
+        const uint64_t s0 = P.seed * 0xA0761D6478BD642Full + (uint64_t)r * 0xE7037ED1A0B428DBull + 1ull + kGolden;
+        uint64_t st = s0 + 2 * kGolden * (uint64_t)lane;
+        int64_t base = 0, hw1 = 0;  // W before the block of 32 steps, h W(1)
+        int64_t lbase = 0;          // !kRing: W(t - h) before the block
+        uint64_t best = 0;
+        int pos = 0;                // ring slot of the block's first step
+        if (kRing) {
+            __syncwarp();  // the previous path's reads
+            if (lane == 0) ring[P.ring - 1] = 0;  // W(0), the slot before step 1
+        }
+        for (int i0 = 1; i0 <= P.nsteps; i0 += 32) {
+            const int i = i0 + lane;
+            const int64_t W = base + warp_scan(increment(st, P, s_ln, s_rec), lane);
+            st += 64 * kGolden;
+            base = __shfl_sync(~0u, W, 31);
+            int64_t lag = 0;
+            if (kRing) {
+                ring[pos + lane] = W;
+                __syncwarp();
+                int s = pos + lane - P.ih;
+                s += s < 0 ? P.ring : 0;
+                lag = ring[s];  // steps before the ring's first lap are not used (i < G)
+                pos += 32;
+                pos = pos == P.ring ? 0 : pos;
+                __syncwarp();
+            } else if (i0 + 31 > P.ih) {
+                const int j = i - P.ih;  // the lagged step
+                const int64_t inc = j >= 1 ? increment(s0 + 2 * kGolden * (uint64_t)(j - 1), P, s_ln, s_rec) : 0;
+                lag = lbase + warp_scan(inc, lane);
+                lbase = __shfl_sync(~0u, lag, 31);
+            }
+            if (i0 + 31 >= P.G) {
+                if (i0 <= P.G) {  // W(1) is in this block
+                    const int64_t w1 = __shfl_sync(~0u, W, P.G - i0);
+                    const uint64_t a = (uint64_t)(w1 < 0 ? -w1 : w1), ha = P.h ? fixedpt::mulhi(a, P.h) : a;
+                    hw1 = w1 < 0 ? -(int64_t)ha : (int64_t)ha;
+                }
+                if (i >= P.G && i <= P.nsteps) {
+                    const int64_t z = W - lag - hw1;
+                    uint64_t v = (uint64_t)(z < 0 ? -z : z);
+                    if (v > best) {  // the boundary's factor, at least 1, only lowers it
+                        if (i > P.ie) v = (uint64_t)((double)v / sqrt(log((double)i / (double)P.G)));
+                        best = v > best ? v : best;
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const uint64_t t = __shfl_xor_sync(~0u, best, o);
+            best = t > best ? t : best;
+        }
+        if (lane == 0) P.stats[r] = (double)best * unit;
+    }
+}
+
+const fixedpt::LogTable& log_table() {
+    static fixedpt::LogTable t;
+    static std::once_flag once;
+    std::call_once(once, [] {
+        for (uint32_t i = 0; i < 256; ++i) t.ln[i] = fixedpt::log_entry(i);
+    });
+    return t;
+}
+
+template <bool kRing>
+cudaError_t launch_paths(const LambdaParams& P, size_t smem, cudaStream_t st) {
+    auto* fn = lambda_paths<kRing>;
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxRingBytes);
+    int dev = 0, sms = 0, per = 0;
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, 32 * kWarps, smem);
+    if (e != cudaSuccess) return e;
+    const int64_t want = ((int64_t)P.reps + kWarps - 1) / kWarps, most = (int64_t)sms * (per < 1 ? 1 : per);
+    fn<<<(unsigned)(want < most ? want : most), 32 * kWarps, smem, st>>>(log_table(), P);
+    return cudaGetLastError();
 }
 
 }  // namespace
@@ -91,9 +194,25 @@ extern "C" bfm_status bfm_lambda(double alpha, double h, double T, int G, int re
     double* d_stats = nullptr;
     cudaError_t e = cudaMallocAsync(&d_stats, sizeof(double) * (size_t)reps, st);
     if (e != cudaSuccess) return cuda_fail(e, "bfm_lambda: cudaMallocAsync");
-    const int block = 128;
-    lambda_paths<<<(reps + block - 1) / block, block, 0, st>>>(h, G, nsteps, ih, reps, seed, d_stats);
-    e = cudaGetLastError();
+    LambdaParams P{};
+    P.G = G;
+    P.nsteps = nsteps;
+    P.ih = ih;
+    P.reps = reps;
+    P.ie = (int)std::min<double>(std::floor(kE * (double)G), 2147483647.0);
+    while ((double)P.ie / (double)G > kE) --P.ie;
+    while (P.ie < nsteps && (double)(P.ie + 1) / (double)G <= kE) ++P.ie;
+    // |W| stays below 13 sqrt(T) (13 standard deviations) and |W - Wlag - h W(1)| below
+    // three times that: the integer part holds 40 sqrt(T)
+    P.frac = 62 - (int)std::ceil(std::log2(40.0 * std::sqrt(T)));
+    P.seed = seed;
+    P.sd = G == 1 ? ~0ull : (uint64_t)std::ldexp(1.0 / std::sqrt((double)G), 64);
+    P.h = h < 1.0 ? (uint64_t)std::ldexp(h, 64) : 0ull;
+    P.stats = d_stats;
+    const int64_t slots = ((int64_t)ih + 63) / 32 * 32;
+    const bool ring = (size_t)slots * kWarps * 8 <= kMaxRingBytes;
+    P.ring = ring ? (int)slots : 0;
+    e = ring ? launch_paths<true>(P, (size_t)slots * kWarps * 8, st) : launch_paths<false>(P, 0, st);
     std::vector<double> stats((size_t)reps);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(stats.data(), d_stats, sizeof(double) * (size_t)reps, cudaMemcpyDeviceToHost, st);
