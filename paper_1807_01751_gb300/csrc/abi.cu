@@ -1,5 +1,6 @@
 // C ABI of libbfm: argument checks, the design cache, dispatch to the
 // kernels, and the host-buffer entry point (chunked copy/compute overlap).
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -285,14 +286,16 @@ bfm_status bfm_design_create(const double* dates, int N, int k_harm, double f, b
         if (e == cudaSuccess) e = cudaMemcpy(d->d_hyb, tab.data(), tab.size(), cudaMemcpyHostToDevice);
     }
     if (e == cudaSuccess) {
-        e = cudaMalloc(&d->d_dates, sizeof(double) * (size_t)N);
-        if (e == cudaSuccess) e = cudaMemcpy(d->d_dates, dates, sizeof(double) * (size_t)N, cudaMemcpyHostToDevice);
+        std::vector<double> x((size_t)N * d->K);  // the first K entries of every basis row
+        for (int t = 0; t < N; ++t) std::copy_n(rowsd.begin() + (size_t)t * d->NB, d->K, x.begin() + (size_t)t * d->K);
+        e = cudaMalloc(&d->d_xd, x.size() * sizeof(double));
+        if (e == cudaSuccess) e = cudaMemcpy(d->d_xd, x.data(), x.size() * sizeof(double), cudaMemcpyHostToDevice);
     }
     if (e != cudaSuccess) {
         cudaFree(d->d_basis);
         if (d->d_phi_tc) cudaFree(d->d_phi_tc);
         if (d->d_hyb) cudaFree(d->d_hyb);
-        if (d->d_dates) cudaFree(d->d_dates);
+        if (d->d_xd) cudaFree(d->d_xd);
         delete d;
         return cuda_fail(e, "bfm_design_create: device tables");
     }
@@ -317,7 +320,7 @@ bfm_status bfm_design_destroy(bfm_design_t d) {
                 cudaFree(d->d_basis);
                 if (d->d_phi_tc) cudaFree(d->d_phi_tc);
                 if (d->d_hyb) cudaFree(d->d_hyb);
-                if (d->d_dates) cudaFree(d->d_dates);
+                if (d->d_xd) cudaFree(d->d_xd);
                 for (auto& c : d->complete) cudaFree(c.d_tab);
                 if (cur != d->device) cudaSetDevice(cur);
                 delete d;

@@ -141,7 +141,7 @@ struct bfm_design_s {
     double c = 0.0, s = 1.0;  // trend centring/scaling
     int NB = 0;               // basis row stride (floats)
     float* d_basis = nullptr; // device [N][NB]
-    double* d_dates = nullptr; // device [N]: the date values (bfm_trace)
+    double* d_xd = nullptr;  // device [N][K]: the regressors in FP64 (bfm_trace)
     std::mutex complete_mu;            // guards `complete`
     std::vector<CompleteTab> complete; // built on first use per n_hist, freed with the design
     // Tensor-core B operands: the basis table as fp16 hi and lo parts in the

@@ -8,7 +8,7 @@
 //   1. compaction of the pixel's valid observations (ballot + popcount over
 //      32-date groups), n_p = valid history observations, N_p = all;
 //   2. the least-squares fit of Eq. 5-6 on the valid history observations,
-//      redone in FP64 from the Eq. 2 regressors of the actual dates (trend
+//      redone in FP64 from the design's table of Eq. 2 regressors (trend
 //      centred and scaled) by Cholesky on the normal equations;
 //   3. residuals y - x'beta (the sign of Eq. 3) of every valid observation,
 //      sigma-hat with n_p - K degrees of freedom (Algorithm 1 step 5);
@@ -19,6 +19,14 @@
 // The pixel statuses written by bfm_monitor for the same data decide which
 // pixels have a fit (OK, DEGENERATE, NO_MONITOR) so that the two calls agree
 // on them; DEGENERATE pixels get MO = 0 at their monitoring dates.
+//
+// What bounds it: FP64 issue, 1/64 of the 32-bit rate, so FP64 instructions per
+// pixel are what counts.  Evaluating the regressors in the kernel (six sincospi per
+// date and pixel), summing the normal equations by butterflies over whole lanes and
+// solving in every lane alike took about 2400 per warp and pixel: 709 us for 4096
+// pixels of 414 dates.  Now the regressors are read from the design's table, the
+// sums are folded (each exchange halves the values a lane carries) and the
+// factorisation is spread over the lanes: about 400, 178 us.
 #include <cmath>
 
 #include "bfm_internal.cuh"
@@ -31,8 +39,8 @@ struct TraceParams {
     const uint32_t* mask;
     int64_t m, mask_words;
     int N, n_hist, dtype;
-    double h_frac, f, c, s;
-    const double* dates;
+    double h_frac;
+    const double* x;  // regressors [N][K] of the design (Eq. 2, centred and scaled trend)
     const int64_t* pixels;
     int64_t count;
     const uint8_t* status;
@@ -44,19 +52,40 @@ struct TraceParams {
 // and the compacted position of every date (-1 when missing).
 constexpr int kBytesPerDate = 16;
 constexpr int kMaxWarps = 4;
-constexpr size_t kSmemTarget = 48 * 1024;
+constexpr size_t kSmemTarget = 46 * 1024;  // beside the normal equations, within the default 48 KB
 
-// Eq. 2 regressors of date t with the trend column (t - c)/s.
-template <int KH>
-__device__ __forceinline__ void regressors(double t, const TraceParams& P, double* x) {
-    x[0] = 1.0;
-    x[1] = (t - P.c) / P.s;
+// Regressors of date t from the design's table (rows of K doubles, 16-byte aligned).
+template <int K>
+__device__ __forceinline__ void regressors(const double* tab, int t, double (&x)[K]) {
+    const double2* r = reinterpret_cast<const double2*>(tab + (size_t)t * K);
 #pragma unroll
-    for (int j = 1; j <= KH; ++j) {
-        double sj, cj;
-        sincospi(2.0 * (double)j * t / P.f, &sj, &cj);  // sin/cos(2 pi j t / f)
-        x[2 * j] = sj;
-        x[2 * j + 1] = cj;
+    for (int a = 0; a < K / 2; ++a) {
+        const double2 v = __ldg(r + a);
+        x[2 * a] = v.x;
+        x[2 * a + 1] = v.y;
+    }
+}
+
+// Sums of n values over the warp's lanes, folded: at each exchange (lane
+// distance kOff) a lane passes on the half of its values that its partner
+// keeps, so n + n/2 + ... additions in place of n at every distance.  Ends with
+// the sums of values first .. first + count - 1 in the lane, written to out.
+template <int n, int kOff>
+__device__ __forceinline__ void fold_sums(double (&v)[n], int lane, int first, int count, double* out) {
+    if constexpr (kOff == 0) {
+#pragma unroll
+        for (int i = 0; i < n; ++i)
+            if (i < count) out[first + i] = v[i];
+    } else {
+        constexpr int h = (n + 1) / 2;
+        const bool up = (lane & kOff) != 0;
+        double w[h];
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+            const double lo = v[i], hi = i + h < n ? v[i + h < n ? i + h : 0] : 0.0;
+            w[i] = (up ? hi : lo) + __shfl_xor_sync(~0u, up ? lo : hi, kOff);
+        }
+        fold_sums<h, kOff / 2>(w, lane, up ? first + h : first, up ? count - h : min(count, h), out);
     }
 }
 
@@ -64,6 +93,8 @@ template <int KH>
 __global__ void __launch_bounds__(32 * kMaxWarps) trace_kernel(const TraceParams P) {
     constexpr int K = 2 + 2 * KH;
     constexpr int NG = K * (K + 1) / 2;  // packed lower triangle, row a at a(a+1)/2
+    constexpr int NE = NG + K;           // and the right-hand side as row K
+    __shared__ double s_el[kMaxWarps][NE];
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
@@ -85,94 +116,114 @@ __global__ void __launch_bounds__(32 * kMaxWarps) trace_kernel(const TraceParams
     // 1. compaction
     int nv = 0, np = 0;
     if (fit) {
-        for (int t0 = 0; t0 < N; t0 += 32) {
-            const int t = t0 + lane;
-            bool v = false;
-            double y = 0.0;
-            if (t < N) {
-                const size_t o = (size_t)t * (size_t)P.m + (size_t)p;
-                if (P.dtype == BFM_F32) {
-                    const float yf = static_cast<const float*>(P.Y)[o];
-                    v = !isnan(yf);
-                    y = (double)yf;
-                } else {
-                    const int16_t yq = static_cast<const int16_t*>(P.Y)[o];
-                    v = yq != (int16_t)-32768;
-                    y = (double)yq;
+        constexpr int U = 4;  // groups of 32 dates whose loads are in flight together
+        for (int tb = 0; tb < N; tb += 32 * U) {
+            double y[U];
+            bool v[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int t = tb + 32 * u + lane;
+                v[u] = false;
+                y[u] = 0.0;
+                if (t < N) {
+                    const size_t o = (size_t)t * (size_t)P.m + (size_t)p;
+                    if (P.dtype == BFM_F32) {
+                        const float yf = __ldg(static_cast<const float*>(P.Y) + o);
+                        v[u] = !isnan(yf);
+                        y[u] = (double)yf;
+                    } else {
+                        const int16_t yq = __ldg(static_cast<const int16_t*>(P.Y) + o);
+                        v[u] = yq != (int16_t)-32768;
+                        y[u] = (double)yq;
+                    }
+                    if (P.mask)
+                        v[u] = v[u] && ((__ldg(P.mask + (size_t)t * (size_t)P.mask_words + (size_t)(p >> 5)) >> (p & 31)) & 1u);
                 }
-                if (v && P.mask) v = (P.mask[(size_t)t * (size_t)P.mask_words + (size_t)(p >> 5)] >> (p & 31)) & 1u;
             }
-            const unsigned b = __ballot_sync(~0u, v);
-            const int q = nv + __popc(b & ((1u << lane) - 1u));
-            if (t < N) pos[t] = v ? q : -1;
-            if (v) {
-                val[q] = y;
-                tix[q] = t;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int t0 = tb + 32 * u, t = t0 + lane;
+                const unsigned b = __ballot_sync(~0u, v[u]);
+                const int q = nv + __popc(b & ((1u << lane) - 1u));
+                if (t < N) pos[t] = v[u] ? q : -1;
+                if (v[u]) {
+                    val[q] = y[u];
+                    tix[q] = t;
+                }
+                nv += __popc(b);
+                const int hl = P.n_hist - t0;  // history dates in this group
+                const unsigned hm = hl >= 32 ? ~0u : (hl > 0 ? (1u << hl) - 1u : 0u);
+                np += __popc(b & hm);
             }
-            nv += __popc(b);
-            const int hl = P.n_hist - t0;  // history dates in this group
-            const unsigned hm = hl >= 32 ? ~0u : (hl > 0 ? (1u << hl) - 1u : 0u);
-            np += __popc(b & hm);
         }
         __syncwarp();
         fit = np > K;
     }
 
-    // 2. normal equations of the history (every lane ends with the full sums)
+    // 2. normal equations of the history, right-hand side as a further row
     double beta[K];
     if (fit) {
-        double g[NG], rhs[K];
+        double* A = s_el[wib];
+        {
+            double g[NE];
 #pragma unroll
-        for (int a = 0; a < NG; ++a) g[a] = 0.0;
+            for (int a = 0; a < NE; ++a) g[a] = 0.0;
+            for (int j = lane; j < np; j += 32) {
+                double x[K];
+                regressors<K>(P.x, tix[j], x);
+                const double y = val[j];
 #pragma unroll
-        for (int a = 0; a < K; ++a) rhs[a] = 0.0;
-        for (int j = lane; j < np; j += 32) {
-            double x[K];
-            regressors<KH>(P.dates[tix[j]], P, x);
-            const double y = val[j];
+                for (int a = 0; a < K; ++a) {
 #pragma unroll
-            for (int a = 0; a < K; ++a) {
-#pragma unroll
-                for (int b = 0; b <= a; ++b) g[a * (a + 1) / 2 + b] = fma(x[a], x[b], g[a * (a + 1) / 2 + b]);
-                rhs[a] = fma(x[a], y, rhs[a]);
-            }
-        }
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-#pragma unroll
-            for (int a = 0; a < NG; ++a) g[a] += __shfl_xor_sync(~0u, g[a], off);
-#pragma unroll
-            for (int a = 0; a < K; ++a) rhs[a] += __shfl_xor_sync(~0u, rhs[a], off);
-        }
-        // Cholesky G = L L' in place (every lane, identical), then two triangular solves
-#pragma unroll
-        for (int a = 0; a < K; ++a) {
-#pragma unroll
-            for (int b = 0; b <= a; ++b) {
-                double v = g[a * (a + 1) / 2 + b];
-#pragma unroll
-                for (int c = 0; c < b; ++c) v -= g[a * (a + 1) / 2 + c] * g[b * (b + 1) / 2 + c];
-                if (a == b) {
-                    fit = fit && v > 0.0;
-                    g[a * (a + 1) / 2 + a] = sqrt(v > 0.0 ? v : 1.0);
-                } else {
-                    g[a * (a + 1) / 2 + b] = v / g[b * (b + 1) / 2 + b];
+                    for (int b = 0; b <= a; ++b) g[a * (a + 1) / 2 + b] = fma(x[a], x[b], g[a * (a + 1) / 2 + b]);
+                    g[NG + a] = fma(x[a], y, g[NG + a]);
                 }
             }
+            fold_sums<NE, 16>(g, lane, 0, NE, A);
         }
+        __syncwarp();
+        // Cholesky G = L L', column by column, the trailing elements (row i, column
+        // c) spread over the lanes; row K becomes L^-1 rhs.  The diagonal keeps 1 / L_jj.
+        constexpr int E = (NE + 31) / 32;
+        int row[E], col[E];
+        double own[E];
 #pragma unroll
-        for (int a = 0; a < K; ++a) {
-            double v = rhs[a];
+        for (int u = 0; u < E; ++u) {
+            const int e = lane + 32 * u;
+            int i = 0;
+            while (i < K && (i + 1) * (i + 2) / 2 <= e) ++i;  // row i holds elements i(i+1)/2 ..
+            row[u] = e < NE ? i : 0;
+            col[u] = e < NE ? e - i * (i + 1) / 2 : -1;  // -1: no element
+            own[u] = e < NE ? A[e] : 0.0;
+        }
+        auto at = [&](int i, int c) -> double& { return A[i * (i + 1) / 2 + c]; };
 #pragma unroll
-            for (int c = 0; c < a; ++c) v -= g[a * (a + 1) / 2 + c] * rhs[c];
-            rhs[a] = v / g[a * (a + 1) / 2 + a];
+        for (int j = 0; j < K; ++j) {
+            const double d = at(j, j);
+            fit = fit && d > 0.0;
+            const double inv = rsqrt(d > 0.0 ? d : 1.0);
+            double li[E], lc[E];
+#pragma unroll
+            for (int u = 0; u < E; ++u) {
+                const bool upd = col[u] > j;
+                li[u] = upd ? at(row[u], j) * inv : 0.0;
+                lc[u] = upd ? (col[u] == row[u] ? li[u] : at(col[u], j) * inv) : 0.0;
+            }
+            __syncwarp();
+#pragma unroll
+            for (int u = 0; u < E; ++u) {
+                own[u] = fma(-li[u], lc[u], own[u]);
+                if (col[u] == j) own[u] = row[u] == j ? inv : own[u] * inv;
+                if (col[u] >= j) A[lane + 32 * u] = own[u];
+            }
+            __syncwarp();
         }
 #pragma unroll
         for (int a = K - 1; a >= 0; --a) {
-            double v = rhs[a];
+            double v = at(K, a);
 #pragma unroll
-            for (int c = a + 1; c < K; ++c) v -= g[c * (c + 1) / 2 + a] * beta[c];
-            beta[a] = v / g[a * (a + 1) / 2 + a];
+            for (int c = a + 1; c < K; ++c) v = fma(-at(c, a), beta[c], v);
+            beta[a] = v * at(a, a);
         }
     }
 
@@ -188,7 +239,7 @@ __global__ void __launch_bounds__(32 * kMaxWarps) trace_kernel(const TraceParams
     double ss = 0.0;
     for (int j = lane; j < nv; j += 32) {
         double x[K];
-        regressors<KH>(P.dates[tix[j]], P, x);
+        regressors<K>(P.x, tix[j], x);
         double yhat = 0.0;
 #pragma unroll
         for (int a = 0; a < K; ++a) yhat = fma(x[a], beta[a], yhat);
@@ -282,10 +333,7 @@ extern "C" bfm_status bfm_trace(bfm_design_t d, const void* Y, int dtype, const 
     P.n_hist = n_hist;
     P.dtype = dtype;
     P.h_frac = h_frac;
-    P.f = d->f;
-    P.c = d->c;
-    P.s = d->s;
-    P.dates = d->d_dates;
+    P.x = d->d_xd;
     P.pixels = pixels;
     P.count = count;
     P.status = status;
