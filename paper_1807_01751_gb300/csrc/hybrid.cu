@@ -2,13 +2,14 @@
 // the per-date scan, the tensor cores for every contraction over dates.
 //
 // A CTA owns 512 pixels (four 128-pixel M-tiles = four TMEM lane sets) and
-// runs one per SM, so that one copy of the basis tables, three 16 KB stages
-// and a residual ring of floor(h_frac n_hist) slots for all 512 pixels share
-// the SM's shared memory.  Warps 0..15 own 32 pixels each (the pixel's TMEM
-// lane is its thread's lane), warp 16 issues the 2-D TMA boxes of Y (128
-// pixels x 8 float or 16 int16 dates, one per M-tile and stage), warp 17
-// issues the tensor-core work and owns the tensor memory.  Per work block of
-// 512 pixels (Section 2.1, Eq. 3-6, Algorithm 1 with missing values masked):
+// runs one per SM, so that one copy of the basis tables, 48 KB of stages and
+// a residual ring of floor(h_frac n_hist) slots for all 512 pixels share the
+// SM's shared memory.  The M-tiles work in two groups of two, each a pipeline
+// of its own over work blocks of 256 pixels: eight pixel warps that own 32
+// pixels each (the pixel's TMEM lane is its thread's lane), a warp that issues
+// the 2-D TMA boxes of Y (128 pixels x 8 float or 16 int16 dates, one per
+// M-tile and stage) and a warp that issues the tensor-core work.  Per work
+// block (Section 2.1, Eq. 3-6, Algorithm 1 with missing values masked):
 //
 //   A   history, 16 dates per chunk: each pixel thread writes its row of the
 //       chunk's A operands into TMEM -- the 0/1 validity mask as fp16 and the
@@ -28,7 +29,7 @@
 //       history observation of its first MOSUM window.  Then delta = G^-1 c,
 //       beta = beta0 + delta, sigma-hat^2 = (s0 - delta'c) / (n_p - K)
 //       (Algorithm 1 step 5), and delta is written as a further A operand.
-//   C   dates from the earliest window start of the tile to N: yhat = X
+//   C   dates from the earliest window start of the block to N: yhat = X
 //       (beta0 + delta) in TMEM pieces; residuals r = y - yhat; history dates
 //       of the first window fill the ring, monitoring dates slide the window
 //       (Eq. 3) and test MO against the boundary of Eq. 4: the exact test
@@ -81,14 +82,31 @@ using namespace stage;
 
 constexpr int kMT = 4;                    // 128-pixel M-tiles per CTA
 constexpr int kPx = 128 * kMT;            // pixels per CTA tile
-constexpr int kCons = 4 * kMT;            // pixel warps
-constexpr int kProdWarp = kCons;          // TMA producer warp
-constexpr int kMmaWarp = kCons + 1;       // tensor-core issuing warp (owns TMEM)
-constexpr int kThreads = 32 * (kCons + 2);
-constexpr int kStages = 3;
+constexpr int kCons = 4 * kMT;            // pixel warps, four per M-tile
 constexpr int kBoxPx = 128;               // TMA box width (one M-tile)
-constexpr int kStageBytes = 16384;        // kMT boxes
-constexpr int kBoxBytes = kStageBytes / kMT;
+constexpr int kBoxBytes = 4096;
+constexpr int kStages = 3;                // stages in flight per group
+// The M-tiles of a CTA work in two groups, each with its own producer and MMA warp,
+// stages and barriers: the four pixel warps of a scheduler then belong to two
+// pipelines, and one computes while the other waits for a stage, an MMA or a solve.
+// With all four M-tiles in one group the kernel issued on 58 % of its cycles, with two
+// groups 68 %: 7.50 -> 6.68 ms (float) and 7.63 -> 6.95 ms (int16) on 8.4 Mi pixels of 414
+// dates, 193 -> 170 us on 250k pixels of 256.  One M-tile per group (24 warps, 80
+// registers) was slower at every size but the smallest.
+constexpr int kGrp = 2;                       // M-tiles per group
+constexpr int kGroups = kMT / kGrp;
+constexpr int kGrpWarps = 4 * kGrp;           // pixel warps of a group
+constexpr int kGrpPx = 128 * kGrp;            // pixels of a group
+constexpr int kStageBytes = kGrp * kBoxBytes; // a stage: kGrp boxes
+constexpr int kProdWarp = kCons;              // first of kGroups TMA producer warps
+constexpr int kMmaWarp = kCons + kGroups;     // first of kGroups MMA warps (it owns TMEM)
+constexpr int kThreads = 32 * (kCons + 2 * kGroups);
+// Stages the loads of one group may lead those of the other.  Every date of a large
+// scene is on a page of its own, and when the groups drift apart the CTA's loads touch
+// more pages than its address translations cover: on the 8.4 Mi-pixel scene 10.1 ms
+// without a limit (int16 13.0), 9.4 at 32 stages (15.4), 6.7 (6.95) at 1 to 8, float also
+// at 16.  Scenes of under 0.5 GB run alike with any limit.
+constexpr int kLead = 4;
 constexpr uint32_t kTmemCols = 512;
 constexpr uint64_t kWaitNs = 2000000000ull;
 constexpr size_t kSmemCap = 232448;       // opt-in dynamic shared memory per block
@@ -133,7 +151,7 @@ struct HybridParams {
 __host__ __device__ inline size_t tab_gram_lo(int npad) { return (size_t)npad * 48; }
 __host__ __device__ inline size_t tab_x(int npad) { return (size_t)npad * 96; }
 __host__ __device__ inline size_t tab_yhat(int npad) { return (size_t)npad * 160; }
-__host__ __device__ inline size_t tab_yhat_bytes(int npad) { return (size_t)npad * 48 + 384; }
+__host__ __device__ inline size_t tab_yhat_bytes(int npad) { return (size_t)npad * 48 + 128; }
 __host__ __device__ inline size_t tab_bytes(int npad) { return tab_yhat(npad) + tab_yhat_bytes(npad); }
 
 struct HLayout {
@@ -170,12 +188,22 @@ __host__ __device__ inline HLayout hyb_layout(int n, int npad, int hmax) {
     L.gl = L.gh + nh16 / 8 * 384;
     L.xt = L.gl + nh16 / 8 * 384;
     L.yh = L.xt + nh16 / 4 * 256;
-    L.stages = up1024(L.yh + tab_yhat_bytes(npad));
-    L.ring = L.stages + (size_t)kStages * kStageBytes;
+    L.stages = L.yh + tab_yhat_bytes(npad);  // every part so far is a multiple of 128 bytes
+    L.ring = L.stages + (size_t)kStages * kMT * kBoxBytes;
     L.bars = L.ring + (size_t)hmax * kPx * 4;
-    L.total = L.bars + (size_t)(2 * kStages + 14) * 8 + 16;
+    // The bound that decides whether a call takes this form counts the tables in full
+    // (256 bytes more), rounds the stages up to 1024 and adds 176 bytes; the barriers
+    // (kBarBytes) fit in what that leaves: yh ends 384 or 896 bytes above a multiple
+    // of 1024, so the three together are 560 bytes or more.
+    L.total = up1024(L.yh + tab_yhat_bytes(npad) + 256) + (size_t)kStages * kMT * kBoxBytes + (size_t)hmax * kPx * 4 + 176;
     return L;
 }
+
+// Barriers: per group 2 kStages + 10, then two for the batch's tables; the TMEM address,
+// the abort flag, a byte per pixel warp and a word per producer.
+constexpr int kGrpBars = 2 * kStages + 10;
+constexpr size_t kBarBytes = (size_t)(kGroups * kGrpBars + 2) * 8 + 8 + kCons + 4 * kGroups;
+static_assert(kBarBytes <= 560, "the barriers fit the slack of hyb_layout's bound");
 
 __device__ __forceinline__ float obs_y(float raw, bool& ok) {
     ok = !isnan(raw);
@@ -267,40 +295,46 @@ __device__ __forceinline__ void raise_abort(volatile uint32_t* abort_flag) {
 }
 
 // Validity of one observation of this thread's pixel: the in-band marker
-// (float NaN, int16 -32768) and, with an explicit mask, the pixel's bit of
-// the date's mask row.  `in_range` false makes the date invalid (and skips
-// the mask read).
+// (float NaN, int16 -32768) and, with an explicit mask, the pixel's mask bit:
+// bit u of `bits` for date u of the group of 8 at hand.  `in_range` false
+// makes the date invalid.
 template <typename T, bool kMask>
 struct Obs {
-    const uint32_t* mp;
-    size_t mws;
-    uint32_t mbit;
-    __device__ __forceinline__ bool valid(T raw, int d, bool in_range) const {
+    uint32_t bits = 0u;
+    __device__ __forceinline__ bool valid(T raw, int u, bool in_range) const {
         bool ok;
         (void)obs_y(raw, ok);
         ok = ok && in_range;
-        if (kMask) ok = ok && in_range && (mp[(size_t)d * mws] & mbit) != 0u;
+        if (kMask) ok = ok && ((bits >> u) & 1u) != 0u;
         return ok;
     }
     // value (0 when invalid) and validity
-    __device__ __forceinline__ float value(T raw, int d, bool in_range, bool& ok) const {
+    __device__ __forceinline__ float value(T raw, int u, bool in_range, bool& ok) const {
         const float y = obs_y(raw, ok);
         ok = ok && in_range;
-        if (kMask) ok = ok && in_range && (mp[(size_t)d * mws] & mbit) != 0u;
+        if (kMask) ok = ok && ((bits >> u) & 1u) != 0u;
         return y;
     }
 };
 
+// Eight dates of a stage into registers: ahead of a wait (for a buffer, for a TMEM load),
+// so that the two latencies overlap.
+template <typename T>
+__device__ __forceinline__ void load8(const T* st, T (&raw)[8]) {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) raw[u] = st[u * kBoxPx];
+}
+
 // Pass A, 8 dates from d8: masked y as tf32 bits, the 0/1 mask as 4 fp16
 // pairs (even date in the low half), and max |y|.
 template <bool kFull, typename T, bool kMask>
-__device__ __forceinline__ void pass_a8(const Obs<T, kMask>& ob, const T* st, int d8, int n, uint32_t* yv,
+__device__ __forceinline__ void pass_a8(const Obs<T, kMask>& ob, const T (&raw)[8], int d8, int n, uint32_t* yv,
                                         uint32_t* mk, float& ymax) {
     float vf[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
         bool ok;
-        float y = ob.value(st[u * kBoxPx], d8 + u, kFull || d8 + u < n, ok);
+        float y = ob.value(raw[u], u, kFull || d8 + u < n, ok);
         y = ok ? y : 0.f;
         ymax = fmaxf(ymax, fabsf(y));
         yv[u] = __float_as_uint(y);
@@ -317,14 +351,14 @@ __device__ __forceinline__ void pass_a8(const Obs<T, kMask>& ob, const T* st, in
 // r0 * s_r split into fp16 hi (11 leading bits) + lo as 4 + 4 packed pairs;
 // with kScan, the date of valid rank `rem` (counted down) becomes wdate.
 template <bool kFull, bool kScan, typename T, bool kMask>
-__device__ __forceinline__ void pass_b8(const Obs<T, kMask>& ob, const T* st, int d8, int n, const float* yh,
+__device__ __forceinline__ void pass_b8(const Obs<T, kMask>& ob, const T (&raw)[8], int d8, int n, const float* yh,
                                         float inv_sb, float s_r, float& ss0, uint32_t* hw, uint32_t* lw, int& rem,
                                         int& wdate) {
     float hi[8], lo[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
         bool ok;
-        const float y = ob.value(st[u * kBoxPx], d8 + u, kFull || d8 + u < n, ok);
+        const float y = ob.value(raw[u], u, kFull || d8 + u < n, ok);
         const float r = ok ? fmaf(-yh[u], inv_sb, y) : 0.f;
         ss0 = fmaf(r, r, ss0);
         const float rs = r * s_r;
@@ -358,12 +392,12 @@ struct Mon {
 
 // History dates [d8, d8 + 8) before n: the first window's residuals into the ring.
 template <typename T, bool kMask>
-__device__ __forceinline__ void mon_hist8(const Obs<T, kMask>& ob, const T* st, int d8, const float* yh,
+__device__ __forceinline__ void mon_hist8(const Obs<T, kMask>& ob, const T (&raw)[8], int d8, const float* yh,
                                           float* ring_t, Mon& mo) {
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
         bool ok;
-        const float y = ob.value(st[u * kBoxPx], d8 + u, true, ok);
+        const float y = ob.value(raw[u], u, true, ok);
         const float r = fmaf(-yh[u], mo.inv_sb, y);
         const bool take = ok && d8 + u >= mo.wdate && mo.slot < mo.fill_end;
         if (take) ring_t[mo.slot] = r;
@@ -392,12 +426,12 @@ __device__ __forceinline__ void mon_step(bool ok, float r, float* ring_t, Mon& m
 
 // Monitoring dates [d8, d8 + 8), all >= n (kFull: all < N).
 template <bool kFull, bool kExt, typename T, bool kMask>
-__device__ __forceinline__ void mon8(const Obs<T, kMask>& ob, const T* st, int d8, int N, const float* yh,
+__device__ __forceinline__ void mon8(const Obs<T, kMask>& ob, const T (&raw)[8], int d8, int N, const float* yh,
                                      float* ring_t, Mon& mo, float (&Wu)[8]) {
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
         bool ok;
-        const float y = ob.value(st[u * kBoxPx], d8 + u, kFull || d8 + u < N, ok);
+        const float y = ob.value(raw[u], u, kFull || d8 + u < N, ok);
         mon_step<kExt>(ok, fmaf(-yh[u], mo.inv_sb, y), ring_t, mo);
         Wu[u] = mo.W;
     }
@@ -405,13 +439,13 @@ __device__ __forceinline__ void mon8(const Obs<T, kMask>& ob, const T* st, int d
 
 // Dates [d8, d8 + 8) that hold n (or N): history dates fill the ring, later ones are monitored.
 template <typename T, bool kMask>
-__device__ __forceinline__ void mon_mixed8(const Obs<T, kMask>& ob, const T* st, int d8, int n, int N,
+__device__ __forceinline__ void mon_mixed8(const Obs<T, kMask>& ob, const T (&raw)[8], int d8, int n, int N,
                                         const float* yh, float* ring_t, Mon& mo, float (&Wu)[8], bool ext) {
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
         const int d = d8 + u;
         bool ok;
-        const float y = ob.value(st[u * kBoxPx], d, d < N, ok);
+        const float y = ob.value(raw[u], u, d < N, ok);
         const float r = fmaf(-yh[u], mo.inv_sb, y);
         if (d < n) {
             const bool take = ok && d >= mo.wdate && mo.slot < mo.fill_end;
@@ -445,24 +479,27 @@ __global__ void __launch_bounds__(kThreads, 1)
     unsigned char* s_yh = smem + Lo.yh;
     unsigned char* stages = smem + Lo.stages;
     float* ring = reinterpret_cast<float*>(smem + Lo.ring);
+    // (the shuffle tells the compiler that the warp index is uniform)
+    const int tid = threadIdx.x, warp = __shfl_sync(~0u, tid >> 5, 0), lane = tid & 31;
+    // the group this warp works for
+    const int g = warp < kCons ? warp / kGrpWarps : (warp - kCons) % kGroups;
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + Lo.bars);
-    uint64_t* full = bars;                  // [kStages] stage landed
-    uint64_t* empty = full + kStages;       // [kStages] stage released by every pixel warp
-    uint64_t* afull = empty + kStages;      // [2] A buffer written by every pixel warp
+    uint64_t* full = bars + g * kGrpBars;   // [kStages] stage landed
+    uint64_t* empty = full + kStages;       // [kStages] stage released by the group's pixel warps
+    uint64_t* afull = empty + kStages;      // [2] A buffer written by the pixel warps
     uint64_t* aempty = afull + 2;           // [2] MMAs reading the A buffer done
     uint64_t* yfull = aempty + 2;           // [2] fitted-value piece computed
-    uint64_t* yempty = yfull + 2;           // [2] fitted-value piece read by every pixel warp
-    uint64_t* accd = yempty + 2;            // pass A sums complete
-    uint64_t* cdone = accd + 1;             // refinement sums complete
-    uint64_t* coefb = cdone + 1;            // coefficient operands written (two uses per block)
-    uint64_t* dminb = coefb + 1;            // earliest window start of the block published
-    uint64_t* finb = dminb + 1;             // the MMA warp's last MMAs done
-    uint64_t* tabb = finb + 1;              // batch: earlier MMAs done / a tile's tables landed
-    uint32_t* s_tmem = reinterpret_cast<uint32_t*>(tabb + 1);
-    int* s_dstart = reinterpret_cast<int*>(s_tmem + 1);  // [2], by block parity
-    volatile uint32_t* abort_flag = s_tmem + 3;
+    uint64_t* yempty = yfull + 2;           // [2] fitted-value piece read by the pixel warps
+    uint64_t* accd = yempty + 2;            // sums complete: pass A, then pass B' (two phases per block)
+    uint64_t* coefb = accd + 1;             // coefficient operands written: beta0, then delta with the window
+                                            // starts published (two phases per block)
+    uint64_t* tabb = bars + kGroups * kGrpBars; // batch: a tile's tables landed
+    uint64_t* tabfree = tabb + 1;           // batch: the MMAs of every group's earlier blocks done
+    uint32_t* s_tmem = reinterpret_cast<uint32_t*>(tabfree + 1);
+    volatile uint32_t* abort_flag = s_tmem + 1;
+    unsigned char* s_dstart = reinterpret_cast<unsigned char*>(s_tmem + 2);  // [kCons] window start / 8 by pixel warp
+    volatile int* s_pos = reinterpret_cast<volatile int*>(s_dstart + kCons);  // [kGroups] stage each producer is at
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if constexpr (!kBatch) {
         const int npad = P.npad;
         const size_t nh16 = (size_t)((P.n + 15) & ~15);
@@ -477,24 +514,26 @@ __global__ void __launch_bounds__(kThreads, 1)
         copy(s_yh, tab_yhat(npad), tab_yhat_bytes(npad));
     }
     if (tid == 0) {
-        for (int s = 0; s < kStages; ++s) {
-            ptx::mbar_init(full + s, 1);
-            ptx::mbar_init(empty + s, kCons);
+        for (int t = 0; t < kGroups; ++t) {
+            uint64_t* b0 = bars + t * kGrpBars;  // in the order of the pointers above
+            const int wpt = kGrpWarps;
+            for (int s = 0; s < kStages; ++s) {
+                ptx::mbar_init(b0 + s, 1);
+                ptx::mbar_init(b0 + kStages + s, wpt);
+            }
+            b0 += 2 * kStages;
+            for (int b = 0; b < 2; ++b) {
+                ptx::mbar_init(b0 + b, wpt);
+                ptx::mbar_init(b0 + 2 + b, 1);
+                ptx::mbar_init(b0 + 4 + b, 1);
+                ptx::mbar_init(b0 + 6 + b, wpt);
+            }
+            ptx::mbar_init(b0 + 8, 1);
+            ptx::mbar_init(b0 + 9, wpt);
         }
-        for (int b = 0; b < 2; ++b) {
-            ptx::mbar_init(afull + b, kCons);
-            ptx::mbar_init(aempty + b, 1);
-            ptx::mbar_init(yfull + b, 1);
-            ptx::mbar_init(yempty + b, kCons);
-        }
-        ptx::mbar_init(accd, 1);
-        ptx::mbar_init(cdone, 1);
-        ptx::mbar_init(coefb, kCons);
-        ptx::mbar_init(dminb, kCons);
-        ptx::mbar_init(finb, 1);
         ptx::mbar_init(tabb, 1);
-        s_dstart[0] = INT_MAX;
-        s_dstart[1] = INT_MAX;
+        ptx::mbar_init(tabfree, kGroups);
+        for (int t = 0; t < kGroups; ++t) s_pos[t] = 0;
         *abort_flag = 0u;
         ptx::fence_mbar_init();
     }
@@ -505,8 +544,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     ptx::tc_fence_after();
     const uint32_t tmem = *s_tmem;
 
-    // 512-pixel work blocks; the tile of block wb and the block's first pixel in it
-    const int64_t nwork = kBatch ? Bt.blocks : (P.m + kPx - 1) / kPx;
+    // Work blocks.  One tile: the pixels of a group, block u of the scene to CTA u % grid,
+    // group (u / grid) % N, so that a scene of few blocks spreads over the SMs first.
+    // Batch: 512 pixels of a tile, a part to each group (the groups share the tile's
+    // tables).
+    const int64_t nwork = kBatch ? Bt.blocks : (P.m + kGrpPx - 1) / kGrpPx;
+    const int64_t wb0 = (int64_t)blockIdx.x + (kBatch ? 0 : (int64_t)gridDim.x * g);
+    const int64_t wstep = kBatch ? (int64_t)gridDim.x : (int64_t)gridDim.x * kGroups;
     auto locate = [&](int64_t wb, int& ti, int64_t& px0) {
         if constexpr (kBatch) {
             int lo = 0, hi = Bt.ntiles - 1;
@@ -518,42 +562,56 @@ __global__ void __launch_bounds__(kThreads, 1)
                     hi = mid - 1;
             }
             ti = lo;
-            px0 = (wb - Bt.tiles[lo].block0) * kPx;
+            px0 = (wb - Bt.tiles[lo].block0) * kPx + g * kGrpPx;
         } else {
             ti = 0;
-            px0 = wb * kPx;
+            px0 = wb * kGrpPx;
         }
     };
-    auto dstart_of = [](int v, int n) -> int {
-        const int d = v < n ? v : n;
-        return d / G * G;
+    // the group's earliest window start, a multiple of the stage's dates
+    auto dstart = [&]() -> int {
+        const volatile uint32_t* w = reinterpret_cast<const volatile uint32_t*>(s_dstart + kGrpWarps * g);
+        uint32_t v = w[0];
+#pragma unroll
+        for (int i = 1; i < kGrp; ++i) v = __vminu4(v, w[i]);
+        const uint32_t a = min(v & 0xffu, (v >> 8) & 0xffu), b = min((v >> 16) & 0xffu, v >> 24);
+        return (int)min(a, b) * 8 / G * G;
     };
 
-    if (warp == kProdWarp) {
+    if (warp >= kProdWarp && warp < kMmaWarp) {
         // ---------------- TMA producer: passes A, B' over the history, C from the window start
         if (lane == 0) {
             if constexpr (!kBatch) ptx::prefetch_tmap(&tmap);
             const uint64_t keep = l2_evict_last(), normal = l2_evict_normal(), drop = l2_evict_first();
-            int64_t js = 0;
+            unsigned char* const st0 = stages + g * (kStages * kStageBytes);
+            int slot = 0;
+            uint32_t lap = 0;  // laps of the ring completed
             bool ok = true;
-            uint32_t dpar = 0;
-            auto issue = [&](const CUtensorMap* tm, int64_t px0, int d0, uint64_t pol) -> bool {
-                const int slot = (int)(js % kStages);
-                if (js >= kStages &&
-                    !wait_released(empty + slot, (uint32_t)(((js / kStages) - 1) & 1), abort_flag, kWaitNs)) {
+            // pos: the stage in the order of blocks, passes and dates.  Waiting for the other
+            // group only keeps the loads together: it ends by itself after 20 us.
+            auto issue = [&](const CUtensorMap* tm, int64_t px0, int d0, uint64_t pol, int pos) -> bool {
+                s_pos[g] = pos;
+                if (s_pos[g ^ 1] < pos - kLead) {
+                    const uint64_t t0 = ptx::globaltimer_ns();
+                    while (s_pos[g ^ 1] < pos - kLead && !*abort_flag && ptx::globaltimer_ns() - t0 < 20000) __nanosleep(50);
+                }
+                if (lap && !wait_released(empty + slot, (lap - 1u) & 1u, abort_flag, kWaitNs)) {
                     raise_abort(abort_flag);
                     return false;
                 }
                 if (*abort_flag) return false;
-                unsigned char* dst = stages + slot * kStageBytes;
                 ptx::mbar_arrive_expect_tx(full + slot, (uint32_t)kStageBytes);
 #pragma unroll
-                for (int g = 0; g < kMT; ++g) tma_box(dst + g * kBoxBytes, tm, full + slot, (int)(px0 + g * kBoxPx), d0, pol);
-                ++js;
+                for (int i = 0; i < kGrp; ++i)
+                    tma_box(st0 + slot * kStageBytes + i * kBoxBytes, tm, full + slot, (int)(px0 + i * kBoxPx), d0, pol);
+                if (++slot == kStages) {
+                    slot = 0;
+                    ++lap;
+                }
                 return true;
             };
-            int it = 0, cur = -1;
-            for (int64_t wb = blockIdx.x; wb < nwork && ok; wb += gridDim.x, ++it) {
+            int cur = -1, pos0 = 0;
+            for (int64_t wb = wb0; wb < nwork && ok; wb += wstep) {
                 int ti;
                 int64_t px0;
                 locate(wb, ti, px0);
@@ -565,30 +623,47 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
                 const HybridParams& Q = kBatch ? Bt.tiles[ti].P : P;
                 const int n = Q.n, N = Q.N;
-                const int nst_h = (n + G - 1) / G;  // stages of one history pass
-                for (int s = 0; s < nst_h && ok; ++s) ok = issue(tm, px0, s * G, keep);
-                for (int s = 0; s < nst_h && ok; ++s) ok = issue(tm, px0, s * G, drop);
+                const int nst = (n + G - 1) / G, per_block = 2 * nst + (N + G - 1) / G;
+                if (px0 >= Q.m) {
+                    pos0 += per_block;
+                    s_pos[g] = pos0;
+                    continue;
+                }
+                for (int d0 = 0; d0 < n && ok; d0 += G) ok = issue(tm, px0, d0, keep, pos0 + d0 / G);
+                for (int d0 = 0; d0 < n && ok; d0 += G) {
+                    // the block's first coefb phase is seen before the last stage of pass B'
+                    // is issued: the second phase cannot complete without that stage
+                    if (d0 + G >= n && !wait_bar(coefb, 0u, abort_flag, kWaitNs)) {
+                        raise_abort(abort_flag);
+                        ok = false;
+                        break;
+                    }
+                    ok = issue(tm, px0, d0, drop, pos0 + nst + d0 / G);
+                }
                 if (!ok) break;
-                if (!wait_bar(dminb, dpar, abort_flag, kWaitNs)) {
+                if (!wait_bar(coefb, 1u, abort_flag, kWaitNs)) {
                     raise_abort(abort_flag);
                     break;
                 }
-                dpar ^= 1u;
-                const int ds = dstart_of(s_dstart[it & 1], n);
-                for (int d0 = ds; d0 < N && ok; d0 += G) ok = issue(tm, px0, d0, normal);
+                for (int d0 = dstart(); d0 < N && ok; d0 += G) ok = issue(tm, px0, d0, normal, pos0 + 2 * nst + d0 / G);
+                pos0 += per_block;
             }
+            s_pos[g] = INT_MAX;
             // copies still in flight land before the CTA's shared memory is released
-            for (int64_t i = js > kStages ? js - kStages : 0; i < js; ++i)
-                ptx::mbar_wait_bounded(full + (i % kStages), (uint32_t)((i / kStages) & 1), kWaitNs);
+            for (int i = 0; i < kStages; ++i) {
+                const uint32_t uses = lap + (i < slot ? 1u : 0u);
+                if (uses) ptx::mbar_wait_bounded(full + i, (uses - 1u) & 1u, kWaitNs);
+            }
         }
         __syncwarp();
-    } else if (warp == kMmaWarp) {
-        // ---------------- tensor-core issuer
+    } else if (warp >= kMmaWarp) {
+        // ---------------- tensor-core issuer of the group
         if (lane == 0) {
             const uint32_t id_g = ptx::idesc_f16(128, 32, false), id_c = ptx::idesc_f16(128, 16, false);
             const uint32_t id_x = ptx::idesc_tf32(128, 16);
             const uint32_t id_y16 = ptx::idesc_f16(128, 16, true), id_y32 = ptx::idesc_f16(128, 32, true);
-            uint32_t cc = 0, pc = 0, cpar = 0;
+            uint32_t cc = 0, pc = 0;
+            uint32_t nacc = 0;  // commits on accd
             bool ok = true;
             // fitted values into piece buffer pc & 1: 16 dates of beta0 in pass B', 32 dates of
             // beta0 + delta in pass C.  Per coefficient set: A_hi x rows 0..15, A_hi x rows 16..31,
@@ -601,8 +676,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const uint64_t y23 = ptx::smem_desc(s_yh + (size_t)(d0 / 8) * 384 + 256, 128, 384);
                 const uint32_t idy = pass_c ? id_y32 : id_y16;
 #pragma unroll
-                for (int g = 0; g < kMT; ++g) {
-                    const uint32_t base = tmem + 128u * g;
+                for (int i = 0; i < kGrp; ++i) {
+                    const uint32_t base = tmem + 128u * (uint32_t)(g * kGrp + i);
                     const uint32_t dcol = pass_c ? base + kColY + 32u * b : base + kColY0 + 16u * b;
                     ptx::mma_f16_ta(dcol, base + kColB0, y01, idy, false);
                     ptx::mma_f16_ta(dcol, base + kColB0 + 8, y23, idy, true);
@@ -623,10 +698,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                 ptx::tc_fence_after();
                 return true;
             };
-            int it = 0, cur = -1;
-            uint32_t tpar = 0;
+            int cur = -1;
+            uint32_t tpar = 0, fpar = 0;
             bool tab_pending = false;  // a table copy not seen to land
-            for (int64_t wb = blockIdx.x; wb < nwork && ok; wb += gridDim.x, ++it) {
+            for (int64_t wb = wb0; wb < nwork && ok; wb += wstep) {
                 int ti;
                 int64_t px0;
                 locate(wb, ti, px0);
@@ -635,27 +710,32 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const int nck = (n + 15) / 16;  // 16-date chunks of the history
                 if constexpr (kBatch) {
                     if (ti != cur) {
-                        // the MMAs of the previous tile have read its tables before they are replaced
-                        if (cur >= 0) {
-                            ptx::mma_commit(tabb);
-                            if (!(ok = wait_bar(tabb, tpar, abort_flag, kWaitNs))) break;
-                            tpar ^= 1u;
+                        // the MMAs of every group's earlier blocks have read the previous
+                        // tile's tables before the first MMA warp replaces them
+                        if (cur >= 0) ptx::mma_commit(tabfree);
+                        if (g == 0) {
+                            if (cur >= 0) {
+                                if (!(ok = wait_bar(tabfree, fpar, abort_flag, kWaitNs))) break;
+                                fpar ^= 1u;
+                            }
+                            const int npad = Q.npad;
+                            const uint32_t bg = (uint32_t)((n + 15) & ~15) / 8 * 384,
+                                           bx = (uint32_t)((n + 15) & ~15) / 4 * 256;
+                            const uint32_t by = (uint32_t)tab_yhat_bytes(npad);
+                            ptx::mbar_arrive_expect_tx(tabb, 2 * bg + bx + by);
+                            ptx::bulk_g2s(s_gh, Q.tabs, bg, tabb);
+                            ptx::bulk_g2s(s_gl, Q.tabs + tab_gram_lo(npad), bg, tabb);
+                            ptx::bulk_g2s(s_xt, Q.tabs + tab_x(npad), bx, tabb);
+                            ptx::bulk_g2s(s_yh, Q.tabs + tab_yhat(npad), by, tabb);
+                            tab_pending = true;
                         }
-                        const int npad = Q.npad;
-                        const uint32_t bg = (uint32_t)((n + 15) & ~15) / 8 * 384, bx = (uint32_t)((n + 15) & ~15) / 4 * 256;
-                        const uint32_t by = (uint32_t)tab_yhat_bytes(npad);
-                        ptx::mbar_arrive_expect_tx(tabb, 2 * bg + bx + by);
-                        ptx::bulk_g2s(s_gh, Q.tabs, bg, tabb);
-                        ptx::bulk_g2s(s_gl, Q.tabs + tab_gram_lo(npad), bg, tabb);
-                        ptx::bulk_g2s(s_xt, Q.tabs + tab_x(npad), bx, tabb);
-                        ptx::bulk_g2s(s_yh, Q.tabs + tab_yhat(npad), by, tabb);
-                        tab_pending = true;
                         if (!(ok = wait_bar(tabb, tpar, abort_flag, kWaitNs))) break;
                         tab_pending = false;
                         tpar ^= 1u;
                         cur = ti;
                     }
                 }
+                if (px0 >= Q.m) continue;
                 // pass A: masked basis sums and X'My
                 for (int c = 0; c < nck && ok; ++c) {
                     if (!(ok = wait_a())) break;
@@ -665,8 +745,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const uint64_t x0 = ptx::smem_desc(s_xt + (size_t)(4 * c) * 256, 256, 128);
                     const uint64_t x1 = ptx::smem_desc(s_xt + (size_t)(4 * c + 2) * 256, 256, 128);
 #pragma unroll
-                    for (int g = 0; g < kMT; ++g) {
-                        const uint32_t base = tmem + 128u * g, a = base + kColA + 24u * b;
+                    for (int i = 0; i < kGrp; ++i) {
+                        const uint32_t base = tmem + 128u * (uint32_t)(g * kGrp + i), a = base + kColA + 24u * b;
                         ptx::mma_f16_ta(base + kColG, a, gh, id_g, c > 0);
                         ptx::mma_f16_ta(base + kColG, a, gl, id_g, true);
                         ptx::mma_tf32_ta(base + kColB, a + 8, x0, id_x, c > 0);
@@ -677,9 +757,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
                 if (!ok) break;
                 ptx::mma_commit(accd);
+                ++nacc;
                 // pass B': fitted values of beta0, refinement sums X'M r0
-                if (!(ok = wait_bar(coefb, cpar, abort_flag, kWaitNs))) break;
-                cpar ^= 1u;
+                if (!(ok = wait_bar(coefb, 0u, abort_flag, kWaitNs))) break;
                 ptx::tc_fence_after();
                 for (int c = 0; c < 2 && c < nck && ok; ++c) ok = piece(16 * c, false);
                 for (int c = 0; c < nck && ok; ++c) {
@@ -688,8 +768,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const uint64_t gh = ptx::smem_desc(s_gh + (size_t)(2 * c) * 384, 384, 128);
                     const uint64_t gl = ptx::smem_desc(s_gl + (size_t)(2 * c) * 384, 384, 128);
 #pragma unroll
-                    for (int g = 0; g < kMT; ++g) {
-                        const uint32_t base = tmem + 128u * g, a = base + kColR + 16u * b;
+                    for (int i = 0; i < kGrp; ++i) {
+                        const uint32_t base = tmem + 128u * (uint32_t)(g * kGrp + i), a = base + kColR + 16u * b;
                         ptx::mma_f16_ta(base + kColC, a, gh, id_c, c > 0);
                         ptx::mma_f16_ta(base + kColC, a + 8, gh, id_c, true);
                         ptx::mma_f16_ta(base + kColC, a, gl, id_c, true);
@@ -700,35 +780,36 @@ __global__ void __launch_bounds__(kThreads, 1)
                     if (c + 2 < nck) ok = piece(16 * (c + 2), false);
                 }
                 if (!ok) break;
-                ptx::mma_commit(cdone);
-                // pass C: fitted values of beta0 + delta from the block's earliest window start
-                if (!(ok = wait_bar(coefb, cpar, abort_flag, kWaitNs))) break;
-                cpar ^= 1u;
+                ptx::mma_commit(accd);
+                ++nacc;
+                // pass C: fitted values of beta0 + delta from the group's earliest window start
+                if (!(ok = wait_bar(coefb, 1u, abort_flag, kWaitNs))) break;
                 ptx::tc_fence_after();
-                const int ds = dstart_of(s_dstart[it & 1], n);
-                for (int d0 = ds; d0 < N && ok; d0 += 32) ok = piece(d0, true);
+                for (int d0 = dstart(); d0 < N && ok; d0 += 32) ok = piece(d0, true);
             }
             if (!ok) raise_abort(abort_flag);
             // a table copy in flight lands before the CTA's shared memory is released
-            if (tab_pending) ptx::mbar_wait_bounded(tabb, tpar, kWaitNs);
+            if (g == 0 && tab_pending) ptx::mbar_wait_bounded(tabb, tpar, kWaitNs);
             // every MMA issued has completed before the tensor memory is released
-            ptx::mma_commit(finb);
-            ptx::mbar_wait_bounded(finb, 0u, kWaitNs);
+            ptx::mma_commit(accd);
+            ptx::mbar_wait_bounded(accd, nacc & 1u, kWaitNs);
         }
         __syncwarp();
     } else {
         // ---------------- pixel warps
-        const int w = warp, g = w >> 2, q = w & 3;
-        const int pl = 32 * w + lane;                       // pixel within the block
+        const int w = warp, q = w & 3;
+        const int pl = 32 * w + lane;                       // ring column of the pixel
         const uint32_t tl = (uint32_t)(32 * q) << 16;       // TMEM lane field of this warp
-        const uint32_t tcol = tmem + 128u * (uint32_t)g;    // this M-tile's columns
+        const uint32_t tcol = tmem + 128u * (uint32_t)(w >> 2);  // this M-tile's columns
+        const int gp = pl % kGrpPx;                         // pixel within the group's block
         float* ring_t = ring + pl;
-        const T* sbase = reinterpret_cast<const T*>(stages + (pl >> 7) * kBoxBytes) + (pl & 127);
+        const T* sbase =
+            reinterpret_cast<const T*>(stages + g * (kStages * kStageBytes) + (gp >> 7) * kBoxBytes) + (pl & 127);
         const float qnan = __int_as_float(0x7fc00000);
         bool bad = false;
         int cslot = 0;
         uint32_t cphase = 0;
-        uint32_t cc = 0, pc = 0, accpar = 0, cdpar = 0, dpar = 0;
+        uint32_t cc = 0, pc = 0;
         // Wait for the next stage and return this thread's column in it.  Fast path:
         // one look at the barrier and a warp vote; the bounded wait (which also ends
         // on the abort flag) only when some lane finds the stage not yet landed.  A
@@ -787,9 +868,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (Q.maxmo) Q.maxmo[p] = qnan;
         };
 
-        int it = 0;
-        int64_t wb = blockIdx.x;
-        for (; wb < nwork; wb += gridDim.x, ++it) {
+        int64_t wb = wb0;
+        for (; wb < nwork; wb += wstep) {
             int ti;
             int64_t px0;
             locate(wb, ti, px0);
@@ -797,17 +877,20 @@ __global__ void __launch_bounds__(kThreads, 1)
             const int n = Q.n, N = Q.N, hmax = Q.hmax;
             const int nck = (n + 15) / 16;  // 16-date chunks of the history
             const int64_t m = Q.m;
-            const int64_t p = px0 + pl;
+            if (px0 >= m) continue;
+            const int64_t p = px0 + gp;
             const bool active = p < m;
-            Obs<T, kMask> ob{kMask ? Q.mask + (active ? (p >> 5) : 0) : nullptr, (size_t)Q.mask_words,
-                             1u << (p & 31)};
+            Obs<T, kMask> ob;
+            // the warp's 32 pixels share one mask word per date
+            const int64_t wcol = (px0 + gp) >> 5;
+            MaskBits mb{kMask ? Q.mask + wcol : nullptr, (size_t)Q.mask_words, kMask && wcol < Q.mask_words ? N : 0};
 
             // ---- pass A: A operands of the masked basis sums and X'My
             float ymax = 0.f;
+            if (kMask) mb.open(0, lane);
             for (int c = 0; c < nck && !bad; ++c) {
                 const uint32_t b = cc & 1u;
-                if (cc >= 2 && !wait_w(aempty + b, ((cc >> 1) - 1) & 1u)) break;
-                ptx::tc_fence_after();
+                if (kMask && (c & 1) == 0) mb.next(16 * c, lane);
                 uint32_t yv[16], mk[8];
                 const T* stg = nullptr;
 #pragma unroll
@@ -816,10 +899,13 @@ __global__ void __launch_bounds__(kThreads, 1)
                     if (d8 < n) {  // warp-uniform: the dates exist
                         if (h == 0 || G == 8) stg = acquire();
                         const T* st = stg + (G == 16 ? h * 8 * kBoxPx : 0);
+                        if (kMask) ob.bits = mb.cur >> (d8 & 31);
+                        T raw[8];
+                        load8(st, raw);
                         if (d8 + 8 <= n)
-                            pass_a8<true>(ob, st, d8, n, yv + 8 * h, mk + 4 * h, ymax);
+                            pass_a8<true>(ob, raw, d8, n, yv + 8 * h, mk + 4 * h, ymax);
                         else
-                            pass_a8<false>(ob, st, d8, n, yv + 8 * h, mk + 4 * h, ymax);
+                            pass_a8<false>(ob, raw, d8, n, yv + 8 * h, mk + 4 * h, ymax);
                         if (G == 8 || h == 1 || d8 + 8 >= n) release();
                     } else {
 #pragma unroll
@@ -829,6 +915,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                 }
                 if (bad) break;
+                if (cc >= 2 && !wait_w(aempty + b, ((cc >> 1) - 1) & 1u)) break;
+                ptx::tc_fence_after();
                 const uint32_t a = tl + tcol + kColA + 24u * b;
                 ptx::tmem_st8(a, mk);
                 ptx::tmem_st16(a + 8, yv);
@@ -837,8 +925,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 ++cc;
             }
             if (bad) break;
-            if (!wait_w(accd, accpar)) break;
-            accpar ^= 1u;
+            if (!wait_w(accd, 0u)) break;
             ptx::tc_fence_after();
             float S[NBR], Bv[K];
             {
@@ -910,16 +997,15 @@ __global__ void __launch_bounds__(kThreads, 1)
             // ---- pass B': r0 = y - yhat0, s0, A operands of X'M r0, the window's start date
             float ss0 = 0.f;
             int rem = wq, wdate = n;
+            if (kMask) mb.open(0, lane);
             for (int c = 0; c < nck && !bad; ++c) {
+                if (kMask && (c & 1) == 0) mb.next(16 * c, lane);
                 if (!wait_w(yfull + (pc & 1u), (pc >> 1) & 1u)) break;
                 ptx::tc_fence_after();
-                float yh[16];
-                ptx::tmem_ld16(tl + tcol + kColY0 + 16u * (pc & 1u), yh);
-                arrive(yempty + (pc & 1u));
-                ++pc;
+                uint32_t yq[2][8];
+                ptx::tmem_ld8_issue(tl + tcol + kColY0 + 16u * (pc & 1u), yq[0]);
+                ptx::tmem_ld8_issue(tl + tcol + kColY0 + 16u * (pc & 1u) + 8u, yq[1]);
                 const uint32_t b = cc & 1u;
-                if (cc >= 2 && !wait_w(aempty + b, ((cc >> 1) - 1) & 1u)) break;
-                ptx::tc_fence_after();
                 uint32_t hw[8], lw[8];
                 const T* stg = nullptr;
 #pragma unroll
@@ -928,21 +1014,33 @@ __global__ void __launch_bounds__(kThreads, 1)
                     if (d8 < n) {
                         if (h == 0 || G == 8) stg = acquire();
                         const T* st = stg + (G == 16 ? h * 8 * kBoxPx : 0);
+                        if (kMask) ob.bits = mb.cur >> (d8 & 31);
+                        T raw[8];
+                        load8(st, raw);
+                        if (h == 0) {
+                            ptx::tmem_wait_ld8(yq[0]);
+                            ptx::tmem_wait_ld8(yq[1]);
+                            arrive(yempty + (pc & 1u));
+                            ++pc;
+                        }
+                        float yh[8];
+#pragma unroll
+                        for (int u = 0; u < 8; ++u) yh[u] = __uint_as_float(yq[h][u]);
                         const bool scan = __any_sync(~0u, rem < 8);  // a pixel may reach its window start
                         const bool fullb = d8 + 8 <= n;
                         if (scan) {
                             if (fullb)
-                                pass_b8<true, true>(ob, st, d8, n, yh + 8 * h, inv_fit, s_r, ss0, hw + 4 * h,
+                                pass_b8<true, true>(ob, raw, d8, n, yh, inv_fit, s_r, ss0, hw + 4 * h,
                                                     lw + 4 * h, rem, wdate);
                             else
-                                pass_b8<false, true>(ob, st, d8, n, yh + 8 * h, inv_fit, s_r, ss0, hw + 4 * h,
+                                pass_b8<false, true>(ob, raw, d8, n, yh, inv_fit, s_r, ss0, hw + 4 * h,
                                                      lw + 4 * h, rem, wdate);
                         } else {
                             if (fullb)
-                                pass_b8<true, false>(ob, st, d8, n, yh + 8 * h, inv_fit, s_r, ss0, hw + 4 * h,
+                                pass_b8<true, false>(ob, raw, d8, n, yh, inv_fit, s_r, ss0, hw + 4 * h,
                                                      lw + 4 * h, rem, wdate);
                             else
-                                pass_b8<false, false>(ob, st, d8, n, yh + 8 * h, inv_fit, s_r, ss0, hw + 4 * h,
+                                pass_b8<false, false>(ob, raw, d8, n, yh, inv_fit, s_r, ss0, hw + 4 * h,
                                                       lw + 4 * h, rem, wdate);
                         }
                         if (G == 8 || h == 1 || d8 + 8 >= n) release();
@@ -955,6 +1053,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                 }
                 if (bad) break;
+                if (cc >= 2 && !wait_w(aempty + b, ((cc >> 1) - 1) & 1u)) break;
+                ptx::tc_fence_after();
                 const uint32_t a = tl + tcol + kColR + 16u * b;
                 ptx::tmem_st8(a, hw);
                 ptx::tmem_st8(a + 8, lw);
@@ -963,8 +1063,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 ++cc;
             }
             if (bad) break;
-            if (!wait_w(cdone, cdpar)) break;
-            cdpar ^= 1u;
+            if (!wait_w(accd, 1u)) break;
             ptx::tc_fence_after();
             float cr[K];
             {
@@ -1038,23 +1137,16 @@ __global__ void __launch_bounds__(kThreads, 1)
                 coef_words<K>(dfin, s_b, wv, rep);
                 coef_store(tl + tcol + kColDl, wv);
             }
-            // the block's earliest window start, for the producer and the MMA warp
+            // the warp's earliest window start, for the producer and the MMA warp (n / 8 <= 224)
             {
-                const unsigned v = active ? (unsigned)wdate : (unsigned)n;
+                const unsigned v = active && wdate < n ? (unsigned)wdate : (unsigned)n;
                 const unsigned wmn = __reduce_min_sync(~0u, v);
-                if (lane == 0) atomicMin(&s_dstart[it & 1], (int)wmn);
+                if (lane == 0) s_dstart[w] = (unsigned char)(wmn >> 3);
             }
             ptx::tmem_wait_st();
-            ptx::tc_fence_before();
-            __syncwarp();
-            if (lane == 0) {
-                mbar_arrive(dminb);
-                mbar_arrive(coefb);
-            }
-            if (!wait_w(dminb, dpar)) break;
-            dpar ^= 1u;
-            const int ds = dstart_of(s_dstart[it & 1], n);
-            if (tid == 0) s_dstart[(it + 1) & 1] = INT_MAX;
+            arrive(coefb);
+            if (!wait_w(coefb, 1u)) break;
+            const int ds = dstart();
 
             // ---- pass C: window fill from the history, then the monitoring scan
             const float inv_scale = (fit && !degenerate) ? 1.f / (sig * sqrtf((float)np)) : 0.f;
@@ -1071,24 +1163,33 @@ __global__ void __launch_bounds__(kThreads, 1)
             int brk = -1;
             float sh = 0.f, sl = 0.f;
             const T* stg = nullptr;
+            if (kMask) mb.open(ds, lane);
             for (int d8 = ds; d8 < N && !bad; d8 += 8) {
                 const int off = d8 - ds;
+                if (kMask) {
+                    if ((off & 31) == 0) mb.next(d8, lane);
+                    ob.bits = mb.cur >> (off & 31);
+                }
                 if ((off & 31) == 0 && !wait_w(yfull + (pc & 1u), (pc >> 1) & 1u)) break;
                 ptx::tc_fence_after();
+                uint32_t yq[8];
+                ptx::tmem_ld8_issue(tl + tcol + kColY + 32u * (pc & 1u) + (uint32_t)(off & 31), yq);
                 if (off % G == 0) {
                     stg = acquire();
                 }
-                const T* st = stg + (off % G);  // dates of the stage are rows of kBoxPx elements
-                const T* st8 = stg + (off % G) * kBoxPx;
-                (void)st;
+                const T* st8 = stg + (off % G) * kBoxPx;  // dates of the stage are rows of kBoxPx elements
+                T raw[8];
+                load8(st8, raw);
+                ptx::tmem_wait_ld8(yq);
                 float yh[8];
-                ptx::tmem_ld8(tl + tcol + kColY + 32u * (pc & 1u) + (uint32_t)(off & 31), yh);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) yh[u] = __uint_as_float(yq[u]);
                 if ((off & 31) == 24 || d8 + 8 >= N) {
                     arrive(yempty + (pc & 1u));
                     ++pc;
                 }
                 if (d8 + 8 <= n) {
-                    mon_hist8(ob, st8, d8, yh, ring_t, mo);
+                    mon_hist8(ob, raw, d8, yh, ring_t, mo);
                 } else {
                     const int J0 = np + 1 + mo.cnt;
                     float Wu[8];
@@ -1096,11 +1197,11 @@ __global__ void __launch_bounds__(kThreads, 1)
                     mo.amax = 0.f;
                     if (d8 >= n && d8 + 8 <= N) {
                         if (maxmo)
-                            mon8<true, true>(ob, st8, d8, N, yh, ring_t, mo, Wu);
+                            mon8<true, true>(ob, raw, d8, N, yh, ring_t, mo, Wu);
                         else
-                            mon8<true, false>(ob, st8, d8, N, yh, ring_t, mo, Wu);
+                            mon8<true, false>(ob, raw, d8, N, yh, ring_t, mo, Wu);
                     } else {
-                        mon_mixed8(ob, st8, d8, n, N, yh, ring_t, mo, Wu, maxmo != nullptr);
+                        mon_mixed8(ob, raw, d8, n, N, yh, ring_t, mo, Wu, maxmo != nullptr);
                     }
                     comp_add(sh, sl, mo.blk);
                     // the boundary grows with the position: a stretch whose largest |MO| stays
@@ -1114,7 +1215,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
                             for (int u = 0; u < 8; ++u) {
                                 const int d = d8 + u;
-                                if (d >= n && ob.valid(st8[u * kBoxPx], d, d < N)) {
+                                if (d >= n && ob.valid(raw[u], u, d < N)) {
                                     const float b2 = Jc > jlimf ? fmaf(lam2ln2, log2_fast(Jc), -blg) : lam2;
                                     if (brk < 0 && fmaf(Wu[u] * Wu[u], inv2, -b2) > 0.f) brk = d;
                                     Jc += 1.f;
@@ -1151,12 +1252,13 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         if (bad) {
             // a wait gave up: mark this thread's unfinished pixels
-            for (; wb < nwork; wb += gridDim.x) {
+            for (; wb < nwork; wb += wstep) {
                 int ti;
                 int64_t px0;
                 locate(wb, ti, px0);
                 const HybridParams& Q = kBatch ? Bt.tiles[ti].P : P;
-                if (px0 + pl < Q.m) write_unfitted(Q, px0 + pl, BFM_PX_TIMEOUT);
+                const int64_t p = px0 + gp;
+                if (p < Q.m) write_unfitted(Q, p, BFM_PX_TIMEOUT);
             }
         }
     }
@@ -1210,8 +1312,8 @@ int hyb_npad(int N) { return (N + 31) / 32 * 32 + 32; }
 //     K-major over dates: (t/4)*256 + (r/8)*128 + (r%8)*16 + (t%4)*4;
 //   fitted values: the K regressors times 2^12 split three ways into fp16 hi
 //     (rows 0..7), mid (8..15) and lo (16..23), read MN-major:
-//     (t/8)*384 + (r/8)*128 + (r%8)*16 + (t%8)*2, plus one group of zeros at
-//     the end (rows 24..31 of the last group are read from it and meet zero
+//     (t/8)*384 + (r/8)*128 + (r%8)*16 + (t%8)*2, plus one row group of zeros
+//     at the end (rows 24..31 of the last group are read from it and meet zero
 //     coefficients).
 void hybrid_tables(const bfm_design_s& d, const std::vector<double>& rows, std::vector<unsigned char>& out) {
     const int npad = hyb_npad(d.N), nbr = 3 + 6 * d.k, K = d.K;
@@ -1334,9 +1436,9 @@ bfm_status launch_hybrid(const bfm_design_s* d, int dtype, const void* Y, const 
     if (!hyb_fill(d, dtype, Y, mask, m, n_hist, h_frac, lambda, brk, mean, sigma, beta, status, maxmo, &P, &tm))
         return BFM_EUNSUPPORTED;
     const int sms = sm_count_cur();
-    const int64_t ntiles = (m + kPx - 1) / kPx;
-    const int grid = (int)(ntiles < (int64_t)sms ? ntiles : (int64_t)sms);
     const size_t smem = hyb_layout(n_hist, P.npad, P.hmax).total;
+    const int64_t nblocks = (m + kGrpPx - 1) / kGrpPx;
+    const int grid = (int)(nblocks < (int64_t)sms ? nblocks : (int64_t)sms);
     if (d->k == 1) return launch_kh<1>(tm, P, dtype, grid, smem, stream);
     if (d->k == 2) return launch_kh<2>(tm, P, dtype, grid, smem, stream);
     return launch_kh<3>(tm, P, dtype, grid, smem, stream);
