@@ -84,7 +84,6 @@ struct MmaParams {
     int N, n_hist, npad, nhpad;  // npad = N padded to 32, nhpad = n_hist padded to 32
     int stages;                   // Y blocks in flight
     int region_bytes;             // table B + A buffers, later the MOSUM ring
-    int vb_extra;                 // bytes of a separate valid-byte area (0: it overlays the delta planes)
     const uint4* phi;             // A_hi, A_lo, B_hi, B_lo (abi.cu tc_tables), each npad dates long
     double h_frac;
     float lambda, c_over_s, inv_s;

@@ -33,11 +33,14 @@
 // Scaling: every A operand row is one pixel, so each thread scales its own
 // rows by powers of two (exact) chosen from its data, keeping fp16 hi + lo
 // splits inside fp16's range; results are scaled back exactly.  TMEM use is
-// 256 columns per CTA and shared memory about 109 KB at 414 dates, so two
-// CTAs share an SM.
+// 256 columns per CTA, so at most two CTAs share an SM, and they do when the
+// tables and the ring leave room: the coefficient operands live in TMEM, the
+// valid bytes beside the A buffers, and the Y ring gives up stages for it
+// (mma_layout).
 #include <cuda_fp16.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <mutex>
@@ -45,6 +48,7 @@
 #include "bfm_internal.cuh"
 #include "ptx.cuh"
 #include "simt_seg.cuh"
+#include "stage.cuh"
 
 namespace bfm {
 
@@ -68,9 +72,12 @@ constexpr int kTile = 128;                  // pixels per CTA
 constexpr int kBlk = 16;                    // dates per Y block (TMA box height) and per A chunk
 constexpr int kPlane = kTile * kBlk * 2;    // bytes of one fp16 A plane (128 x 16)
 constexpr int kBufBytes = 3 * kPlane;       // one A buffer (three planes)
-constexpr int kMaxStages = 8;
-constexpr int kCoefPlane = kTile * 16 * 2;  // one [128 x 16] coefficient plane
-constexpr uint32_t kColG = 0, kColB = 32, kColC = 48, kColY = 64;
+constexpr int kMaxStages = 6;
+constexpr int kPairs = kTile / 32;           // warp pairs (w, w + 4)
+// TMEM columns: basis sums [0, 32), X'My [32, 48), X'M r0 [48, 64), fitted values [64, 256).
+// The basis sums are dead after the solve: beta0 hi, lo and delta hi, lo ([128 x 16]
+// fp16 A operands, 8 columns each) take their place.
+constexpr uint32_t kColG = 0, kColB = 32, kColC = 48, kColY = 64, kColBeta = 0, kColDelta = 16;
 constexpr int kPiece = 192;                 // fitted-value dates per TMEM piece
 constexpr uint32_t kTmemCols = 256;         // 64 + kPiece: two CTAs fit one SM's TMEM
 constexpr uint64_t kWaitNs = 2000000000ull;
@@ -129,19 +136,17 @@ __device__ __forceinline__ void mma_kb(uint32_t dcol, const unsigned char* aplan
     ptx::mma_f16(dcol, ad, bd, ptx::idesc_f16(kTile, 16, false), acc);
 }
 
-// X c over dates [d0, d0 + n) into TMEM column dcol: A = [c_hi | 0], [c_lo | 0]
-// (K = 16 coefficient slots), B = table A read MN-major (N = dates): K-direction
+// X c over dates [d0, d0 + n) into TMEM column dcol: A = [c_hi | 0] at TMEM column
+// ccol and [c_lo | 0] 8 columns on (K = 16 coefficient slots), B = table A read MN-major (N = dates): K-direction
 // (row-group) stride 128 B, N-direction (date-group) stride 256 B.
-__device__ __forceinline__ void mma_xc(uint32_t dcol, const unsigned char* chi, const unsigned char* clo,
-                                       const unsigned char* tab_hi, const unsigned char* tab_lo, int d0, int n,
-                                       bool accumulate) {
-    const uint64_t ah = ptx::smem_desc(chi, kALbo, 128), al = ptx::smem_desc(clo, kALbo, 128);
+__device__ __forceinline__ void mma_xc(uint32_t dcol, uint32_t ccol, const unsigned char* tab_hi,
+                                       const unsigned char* tab_lo, int d0, int n, bool accumulate) {
     const uint32_t id = ptx::idesc_f16(kTile, n, true);
     const uint64_t bh = ptx::smem_desc(tab_hi + (size_t)(d0 / 8) * kTabLbo, 128, kTabLbo);
     const uint64_t bl = ptx::smem_desc(tab_lo + (size_t)(d0 / 8) * kTabLbo, 128, kTabLbo);
-    ptx::mma_f16(dcol, ah, bh, id, accumulate);
-    ptx::mma_f16(dcol, al, bh, id, true);
-    ptx::mma_f16(dcol, ah, bl, id, true);
+    ptx::mma_f16_ta(dcol, ccol, bh, id, accumulate);
+    ptx::mma_f16_ta(dcol, ccol + 8, bh, id, true);
+    ptx::mma_f16_ta(dcol, ccol, bl, id, true);
 }
 
 template <typename T>
@@ -207,21 +212,22 @@ __device__ __forceinline__ void mma_block(const CUtensorMap* tmap, const MmaPara
     unsigned char* tB_hi = region;
     unsigned char* tB_lo = tB_hi + tb;
     unsigned char* sA = tB_lo + tb;
-    unsigned char* sC = region + P.region_bytes;  // beta0 hi, beta0 lo, delta hi, delta lo planes
-    unsigned char* sY = sC + 4 * kCoefPlane;      // Y blocks [16 dates][128 px]
+    unsigned char* sY = region + P.region_bytes;  // Y blocks [16 dates][128 px]
     const int S = P.stages;
-    // per-chunk valid bytes [nbh][2][128], then a float per thread: in the delta
-    // planes (free until the delta is known) when they fit there, else after the stages
-    unsigned char* sVb = P.vb_extra ? sY + (size_t)S * kStageBytes : sC + 2 * kCoefPlane;
+    // in the region behind the A buffers, until the MOSUM ring takes it: per-chunk
+    // valid bytes [nbh][2][128], then a float per thread
+    unsigned char* sVb = sA + 2 * kBufBytes;
     float* sX = reinterpret_cast<float*>(sVb + (size_t)((P.n_hist + kBlk - 1) / kBlk) * 2 * kTile);
-    uint64_t* bars = reinterpret_cast<uint64_t*>(sY + (size_t)S * kStageBytes + P.vb_extra);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(sY + (size_t)S * kStageBytes);
     uint64_t* bar_buf = bars + 0;  // [2] A-buffer reuse
     uint64_t* bar_done = bars + 2;
     uint64_t* full = bars + 3;                 // [S] Y block landed
-    uint64_t* empty = bars + 3 + kMaxStages;   // [S] Y block released (256 arrivals)
-    uint64_t* rdy = bars + 3 + 2 * kMaxStages;  // [2] MOSUM group published by the first threads
-    uint64_t* cons = rdy + 2;                    // [2] MOSUM group consumed by the second threads
-    int* s_dstart = reinterpret_cast<int*>(cons + 2);
+    uint64_t* empty = bars + 3 + kMaxStages;   // [S] Y block released (kPairs arrivals)
+    // the two warps of a pair hand MOSUM groups to each other, one arrival a group
+    uint64_t* rdy = bars + 3 + 2 * kMaxStages + 4 * ((threadIdx.x >> 5) & (kPairs - 1));  // [2] published by the first warp
+    uint64_t* cons = rdy + 2;                                                             // [2] consumed by the second
+    uint64_t* afull = bars + 3 + 2 * kMaxStages + 4 * kPairs;  // [2] A buffer written by every warp
+    int* s_dstart = reinterpret_cast<int*>(afull + 2);
 
     const int tid = threadIdx.x, warp = tid >> 5;
     const int px = tid & (kTile - 1), half = tid >> 7;
@@ -235,12 +241,10 @@ __device__ __forceinline__ void mma_block(const CUtensorMap* tmap, const MmaPara
         for (int i = 0; i < 3; ++i) ptx::mbar_init(bars + i, 1);
         for (int i = 0; i < S; ++i) {
             ptx::mbar_init(full + i, 1);
-            ptx::mbar_init(empty + i, kThreads);
+            ptx::mbar_init(empty + i, kPairs);
         }
-        for (int i = 0; i < 2; ++i) {
-            ptx::mbar_init(rdy + i, kTile);
-            ptx::mbar_init(cons + i, kTile);
-        }
+        for (int i = 0; i < 4 * kPairs; ++i) ptx::mbar_init(rdy + i, 1);  // thread 0's pair is the first
+        for (int i = 0; i < 2; ++i) ptx::mbar_init(afull + i, kThreads / 32);
         ptx::fence_mbar_init();
         *s_dstart = N;
         ptx::prefetch_tmap(tmap);
@@ -267,13 +271,16 @@ __device__ __forceinline__ void mma_block(const CUtensorMap* tmap, const MmaPara
     bool ok = true;
 
     const uint64_t keep = l2_policy_evict_last(), last = l2_policy_evict_first();
-    const uint32_t* mrow = P.mask + (p0 >> 5) + (px >> 5);
+    // the warp's 32 pixels share one mask word per date
+    const int64_t wcol = (p0 >> 5) + (px >> 5);
+    stage::MaskBits mb{kMask ? P.mask + wcol : nullptr, (size_t)P.mask_words, kMask && wcol < P.mask_words ? N : 0};
+    const int lane = tid & 31;
 
     // ---- Y stream: passes over date blocks [b0, b1) -------------------------------------------
     // Block q of the kernel's sequence sits in stage q % S; the producer
     // thread keeps S blocks in flight and refills a stage once its empty
-    // barrier has seen 256 arrivals (the producer's 256 after a chunk barrier
-    // in the history passes, 2 from each first thread in the MOSUM pass).
+    // barrier has seen kPairs arrivals (the producer's once a chunk is written in
+    // the history passes, one from each first warp in the MOSUM pass).
     uint32_t q_next = 0, s_q0 = 0;
     int s_b0 = 0, s_b1 = 0, s_tlim = 0;
     int producer = 0;  // thread 0 in the history passes, thread 128 in the MOSUM pass
@@ -311,8 +318,9 @@ __device__ __forceinline__ void mma_block(const CUtensorMap* tmap, const MmaPara
         if (bd + S < s_b1) issue(q + (uint32_t)S, bd + S);
     };
     // dates [t0, t0 + 8) of this pixel from a waited stage: values (0 where
-    // invalid) and valid bits (missing, masked, t >= tlim, pixel beyond m)
-    auto read8 = [&](const unsigned char* sb, int t0, float (&y)[8]) -> uint32_t {
+    // invalid) and valid bits (missing, masked, t >= tlim, pixel beyond m);
+    // mbits: the pixel's mask bits of these dates
+    auto read8 = [&](const unsigned char* sb, int t0, uint32_t mbits, float (&y)[8]) -> uint32_t {
         const int r0 = t0 & (kBlk - 1);
         const int nt = s_tlim - t0;  // dates of the group before tlim
         const uint32_t lim = !active || nt <= 0 ? 0u : (nt >= 8 ? 0xffu : (1u << nt) - 1u);
@@ -324,26 +332,50 @@ __device__ __forceinline__ void mma_block(const CUtensorMap* tmap, const MmaPara
             vb |= (v ? 1u : 0u) << e;
         }
         vb &= lim;
-        if constexpr (kMask) {
-#pragma unroll
-            for (int e = 0; e < 8; ++e)
-                if ((vb >> e) & 1u)
-                    vb &= ~((((__ldg(mrow + (size_t)(t0 + e) * P.mask_words) >> (px & 31)) & 1u) ^ 1u) << e);
-        }
+        if constexpr (kMask) vb &= mbits;
 #pragma unroll
         for (int e = 0; e < 8; ++e) y[e] = ((vb >> e) & 1u) ? y[e] : 0.f;
         return vb;
     };
-    // history passes: after the chunk's barrier every thread is done with
-    // block c, so thread 0 completes its empty phase at once and refills it
+    // the same as integers (int16 storage)
+    auto read8i = [&](const unsigned char* sb, int t0, uint32_t mbits, int (&y)[8]) -> uint32_t {
+        const int r0 = t0 & (kBlk - 1);
+        const int nt = s_tlim - t0;
+        uint32_t vb = !active || nt <= 0 ? 0u : (nt >= 8 ? 0xffu : (1u << nt) - 1u);
+        if constexpr (kMask) vb &= mbits;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const int v = reinterpret_cast<const int16_t*>(sb)[(r0 + e) * kTile + px];
+            const bool ok = v != -32768 && ((vb >> e) & 1u);
+            y[e] = ok ? v : 0;
+            vb = ok ? vb : vb & ~(1u << e);
+        }
+        return vb;
+    };
+    // history passes: when a chunk is written every thread is done with block
+    // c, so thread 0 completes its empty phase at once and refills it
     auto chunk_release = [&](int bd) {
         if (tid == producer) {
-            block_release(bd, kThreads);
+            block_release(bd, kPairs);
             block_refill(bd);
         }
     };
 
     uint32_t done_uses = 0, buf_uses[2] = {0u, 0u};
+    // A buffer `buf` of chunk c is written: every warp says so and goes on, thread 0 waits
+    // for all of them (which are then also done with Y block c) before it issues the
+    // chunk's MMAs.  A CTA barrier per chunk cost 1.7 stall cycles per instruction here.
+    auto chunk_written = [&](int c, int buf) {
+        ptx::fence_async_smem();
+        ptx::tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(afull + buf);
+        if (tid == 0) {
+            ok &= ptx::mbar_wait_bounded(afull + buf, buf_uses[buf] & 1u, kWaitNs);
+            ptx::tc_fence_after();
+            chunk_release(c);
+        }
+    };
     auto wait_done = [&]() {
         ok &= ptx::mbar_wait_bounded(bar_done, done_uses & 1u, kWaitNs);
         ++done_uses;
@@ -375,8 +407,12 @@ __device__ __forceinline__ void mma_block(const CUtensorMap* tmap, const MmaPara
     for (int attempt = 0; attempt < 2; ++attempt) {
         open(0, nbh, n_hist, keep);
         float ym = 0.f;
+        int yim = 0;
+        if (kMask) mb.open(0, lane);
         for (int c = 0; c < nbh; ++c) {
             const int buf = c & 1;
+            if (kMask && !(c & 1)) mb.next(c * kBlk, lane);
+            const uint32_t mk16 = mb.cur >> ((c & 1) * kBlk);  // the chunk's mask bits
             unsigned char* pl = sA + (size_t)buf * kBufBytes;
             acquire(buf);
             const unsigned char* sb = block_wait(c);
@@ -385,7 +421,7 @@ __device__ __forceinline__ void mma_block(const CUtensorMap* tmap, const MmaPara
 #pragma unroll
                 for (int g = 0; g < 2; ++g) {
                     float yg[8];
-                    read8(sb, c * kBlk + g * 8, yg);
+                    read8(sb, c * kBlk + g * 8, mk16 >> (g * 8), yg);
                     float gm = 0.f;
 #pragma unroll
                     for (int e = 0; e < 8; ++e) gm = fmaxf(gm, fabsf(yg[e]));
@@ -395,31 +431,28 @@ __device__ __forceinline__ void mma_block(const CUtensorMap* tmap, const MmaPara
                     }
                 }
             }
-            const uint32_t vc = read8(sb, c * kBlk + half * 8, yc);
+            int yi[8];
+            const uint32_t vc = kInt ? read8i(sb, c * kBlk + half * 8, mk16 >> (half * 8), yi)
+                                     : read8(sb, c * kBlk + half * 8, mk16 >> (half * 8), yc);
             float mk[8], a1[8], a2[8];
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
                 const bool v = (vc >> e) & 1u;
                 mk[e] = v ? 1.f : 0.f;
-                const float y = yc[e];
-                ym = fmaxf(ym, fabsf(y));
                 if constexpr (kInt) {
-                    const int yi = (int)y;
-                    a1[e] = (float)((yi >> 8) * 256);
-                    a2[e] = (float)(yi & 255);
+                    yim = max(yim, abs(yi[e]));
+                    a1[e] = (float)(yi[e] & ~255);
+                    a2[e] = (float)(yi[e] & 255);
                 } else {
-                    split_hi_lo(y * s_y, a1[e], a2[e]);
+                    ym = fmaxf(ym, fabsf(yc[e]));
+                    split_hi_lo(yc[e] * s_y, a1[e], a2[e]);
                 }
             }
             st_a(pl, px, half, mk);
             st_a(pl + kPlane, px, half, a1);
             st_a(pl + 2 * kPlane, px, half, a2);
-            ptx::fence_async_smem();
-            ptx::tc_fence_before();
-            __syncthreads();
-            chunk_release(c);
+            chunk_written(c, buf);
             if (tid == 0) {
-                ptx::tc_fence_after();
                 const int d0 = c * kBlk;
                 const bool first = c == 0;
                 mma_kb(tmem + kColG, pl, 0, tA_hi, d0, !first);
@@ -438,6 +471,7 @@ __device__ __forceinline__ void mma_block(const CUtensorMap* tmap, const MmaPara
             ++buf_uses[buf];
         }
         wait_done();
+        if (kInt) ym = (float)yim;
         ymax = fmaxf(ym, pair_exchange(ym));
         if (kInt) break;
         const float qy = ymax * s_y;
@@ -477,20 +511,27 @@ __device__ __forceinline__ void mma_block(const CUtensorMap* tmap, const MmaPara
         s_b = pow2_scale(bm, 12);
         s_r = pow2_scale(ymax + bsum, 12);
     }
-    auto write_coef = [&](const float (&coef)[K], unsigned char* hi_plane, unsigned char* lo_plane) {
-        float h[8], l[8], z[8];
+    auto write_coef = [&](const float (&coef)[K], uint32_t col) {
+        float h[8], l[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const float cs = i < K ? coef[i] * s_b : 0.f;
             split_hi_lo(cs, h[i], l[i]);
-            z[i] = 0.f;
         }
-        st_a(hi_plane, px, 0, h);
-        st_a(hi_plane, px, 1, z);
-        st_a(lo_plane, px, 0, l);
-        st_a(lo_plane, px, 1, z);
+        uint32_t w[16];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            w[j] = pack_h2(h[2 * j], h[2 * j + 1]);
+            w[8 + j] = pack_h2(l[2 * j], l[2 * j + 1]);
+            w[4 + j] = w[12 + j] = 0u;
+        }
+        ptx::tmem_st16(tmem + lane_base + col, w);
+        ptx::tmem_wait_st();
     };
-    if (half == 0) write_coef(beta, sC, sC + kCoefPlane);
+    ptx::tc_fence_before();
+    __syncthreads();  // the basis sums read by both threads of the pair before beta0 takes their columns
+    ptx::tc_fence_after();
+    if (half == 0) write_coef(beta, kColBeta);
     const float inv_b = 1.f / s_b;
 
     // ---- one refinement step: r0 = y - X beta0 on the history, c = X'M r0 ------------------
@@ -499,6 +540,7 @@ __device__ __forceinline__ void mma_block(const CUtensorMap* tmap, const MmaPara
     // group's valid bits.
     float ss = 0.f;
     open(0, nbh, n_hist, keep);
+    if (kMask) mb.open(0, lane);
     for (int d0 = 0; d0 < nbh * kBlk; d0 += kPiece) {
         const int w = nbh * kBlk - d0 < kPiece ? nbh * kBlk - d0 : kPiece;
         ptx::fence_async_smem();
@@ -506,7 +548,7 @@ __device__ __forceinline__ void mma_block(const CUtensorMap* tmap, const MmaPara
         __syncthreads();  // coefficient planes written; previous piece's TMEM reads done
         if (tid == 0) {
             ptx::tc_fence_after();
-            mma_xc(tmem + kColY, sC, sC + kCoefPlane, tA_hi, tA_lo, d0, w, false);
+            mma_xc(tmem + kColY, tmem + kColBeta, tA_hi, tA_lo, d0, w, false);
             ptx::mma_commit(bar_done);
         }
         wait_done();
@@ -520,7 +562,8 @@ __device__ __forceinline__ void mma_block(const CUtensorMap* tmap, const MmaPara
             acquire(buf);
             float yc[8], yh[8];
             const unsigned char* sb = block_wait(c);
-            const uint32_t vc = read8(sb, t0, yc);
+            if (kMask && !(c & 1)) mb.next(c * kBlk, lane);
+            const uint32_t vc = read8(sb, t0, mb.cur >> ((c & 1) * kBlk + half * 8), yc);
             ptx::tmem_wait_ld8(rq);
 #pragma unroll
             for (int e = 0; e < 8; ++e) yh[e] = __uint_as_float(rq[e]);
@@ -536,12 +579,8 @@ __device__ __forceinline__ void mma_block(const CUtensorMap* tmap, const MmaPara
             sVb[(c * 2 + half) * kTile + px] = (unsigned char)vc;
             st_a(pl, px, half, rh);
             st_a(pl + kPlane, px, half, rl);
-            ptx::fence_async_smem();
-            ptx::tc_fence_before();
-            __syncthreads();
-            chunk_release(c);
+            chunk_written(c, buf);
             if (tid == 0) {
-                ptx::tc_fence_after();
                 const int dd = c * kBlk;
                 const bool first = c == 0;
                 mma_kb(tmem + kColC, pl, 0, tA_hi, dd, !first);
@@ -594,8 +633,7 @@ __device__ __forceinline__ void mma_block(const CUtensorMap* tmap, const MmaPara
         scale = sigma * sqrtf((float)n_i);
         jlim = (int)floor(kEuler * (double)n_i);
     }
-    __syncthreads();  // valid bytes read by both threads before the delta planes overwrite them
-    if (half == 0) write_coef(dl, sC + 2 * kCoefPlane, sC + 3 * kCoefPlane);
+    if (half == 0) write_coef(dl, kColDelta);
     const bool degenerate = !(sigma > kDegenerateRatio * ymax) || ymax == 0.f;
     // The MOSUM pass starts at the earliest such date over the tile's pixels
     // that get a break test (prefix sums from there on differ from those
@@ -633,6 +671,7 @@ __device__ __forceinline__ void mma_block(const CUtensorMap* tmap, const MmaPara
     uint32_t grp = 0;  // MOSUM group sequence number (the same in both threads)
     producer = kTile;  // the second threads trail the first ones: refills stay off the first threads' path
     open(d_start / kBlk, nball, N, last);
+    if (kMask && half == 0) mb.open(d_start, lane);
     for (int d0 = d_start; d0 < P.npad; d0 += kPiece) {
         const int w = P.npad - d0 < kPiece ? P.npad - d0 : kPiece;
         ptx::fence_async_smem();
@@ -640,8 +679,8 @@ __device__ __forceinline__ void mma_block(const CUtensorMap* tmap, const MmaPara
         __syncthreads();
         if (tid == 0) {
             ptx::tc_fence_after();
-            mma_xc(tmem + kColY, sC, sC + kCoefPlane, tA_hi, tA_lo, d0, w, false);
-            mma_xc(tmem + kColY, sC + 2 * kCoefPlane, sC + 3 * kCoefPlane, tA_hi, tA_lo, d0, w, true);
+            mma_xc(tmem + kColY, tmem + kColBeta, tA_hi, tA_lo, d0, w, false);
+            mma_xc(tmem + kColY, tmem + kColDelta, tA_hi, tA_lo, d0, w, true);
             ptx::mma_commit(bar_done);
         }
         wait_done();
@@ -655,8 +694,12 @@ __device__ __forceinline__ void mma_block(const CUtensorMap* tmap, const MmaPara
                 float yc[8], yh[8];
                 const int bd = c0 / kBlk;
                 if ((c0 & 8) == 0) sb = block_wait(bd);
-                const uint32_t vb = read8(sb, c0, yc);
-                if (c0 & 8) block_release(bd, 2);
+                if (kMask && !((c0 - d_start) & 31)) mb.next(c0, lane);
+                const uint32_t vb = read8(sb, c0, mb.cur >> ((c0 - d_start) & 31), yc);
+                if (c0 & 8) {
+                    __syncwarp();
+                    if (lane == 0) block_release(bd, 1);
+                }
                 ptx::tmem_wait_ld8(rq);
 #pragma unroll
                 for (int e = 0; e < 8; ++e) yh[e] = __uint_as_float(rq[e]);
@@ -680,23 +723,28 @@ __device__ __forceinline__ void mma_block(const CUtensorMap* tmap, const MmaPara
                     Sh = t;
                 }
                 if (grp >= 2) ok &= ptx::mbar_wait_bounded(cons + (grp & 1), ((grp >> 1) - 1u) & 1u, kWaitNs);
+                // the slots are counted along (a popcount per date issues at an eighth of the rate)
+                mbox[(grp & 1) * kTile + px] = ((uint32_t)slot << 8) | vb;
                 if (slot <= R - 8) {  // the group's slots do not wrap
                     float* wp = ring + slot * kTile + px;
 #pragma unroll
                     for (int e = 0; e < 8; ++e)
-                        if ((vb >> e) & 1u) wp[__popc(vb & ((1u << e) - 1u)) * kTile] = Sv[e];
+                        if ((vb >> e) & 1u) {
+                            *wp = Sv[e];
+                            wp += kTile;
+                            ++slot;
+                        }
+                    slot -= slot >= R ? R : 0;
                 } else {
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) {
-                        int se = slot + __popc(vb & ((1u << e) - 1u));
-                        se -= se >= R ? R : 0;
-                        if ((vb >> e) & 1u) ring[se * kTile + px] = Sv[e];
-                    }
+                    for (int e = 0; e < 8; ++e)
+                        if ((vb >> e) & 1u) {
+                            ring[slot * kTile + px] = Sv[e];
+                            slot = slot + 1 == R ? 0 : slot + 1;
+                        }
                 }
-                mbox[(grp & 1) * kTile + px] = ((uint32_t)slot << 8) | vb;
-                slot += __popc(vb);
-                slot -= slot >= R ? R : 0;
-                mbar_arrive(rdy + (grp & 1));
+                __syncwarp();
+                if (lane == 0) mbar_arrive(rdy + (grp & 1));
             }
         } else {
 #pragma unroll 1
@@ -709,21 +757,21 @@ __device__ __forceinline__ void mma_block(const CUtensorMap* tmap, const MmaPara
                     const uint32_t vb = word & 0xffu, mv = vb & mon;
                     const int sl0 = (int)(word >> 8);
                     float wv[8], mo2[8];
-                    const bool nowrap = sl0 <= R - 8 && sl0 >= h;  // neither the slots nor their lags wrap
+                    // slot of the next valid date and the slot h behind it, both in [0, R) (at an
+                    // invalid date they may hold anything: nothing of it is used)
+                    int se = sl0, ls = sl0 - h;
+                    ls += ls < 0 ? R : 0;
 #pragma unroll
                     for (int e = 0; e < 8; ++e) {
-                        int se = sl0 + __popc(vb & ((1u << e) - 1u));
-                        int ls = se - h;
-                        if (!nowrap) {
-                            se -= se >= R ? R : 0;
-                            ls = se - h;
-                            ls += ls < 0 ? R : 0;
-                        }
                         const float W = ring[se * kTile + px] - ring[ls * kTile + px];
                         const float mo = W * inv_scale;
                         const bool mm = (mv >> e) & 1u;
                         wv[e] = mm ? W : 0.f;
                         mo2[e] = mm ? mo * mo : 0.f;
+                        if ((vb >> e) & 1u) {
+                            se = se + 1 == R ? 0 : se + 1;
+                            ls = ls + 1 == R ? 0 : ls + 1;
+                        }
                     }
                     // log+ >= 1: |MO| <= lambda never crosses; the exact boundary
                     // only for candidates before the first crossing
@@ -752,7 +800,8 @@ __device__ __forceinline__ void mma_block(const CUtensorMap* tmap, const MmaPara
                     const float gsum = ((wv[0] + wv[1]) + (wv[2] + wv[3])) + ((wv[4] + wv[5]) + (wv[6] + wv[7]));
                     comp_add(m0, m0c, gsum);
                 }
-                mbar_arrive(cons + (grp & 1));
+                __syncwarp();
+                if (lane == 0) mbar_arrive(cons + (grp & 1));
                 if (tid == producer && (c0 & 8)) block_refill(c0 / kBlk);
             }
         }
@@ -831,29 +880,45 @@ int ring_len(int n_hist, double h_frac) {
 }
 
 struct MmaLayout {
-    int stages, region_bytes, vb_extra;
+    int stages, region_bytes;
     size_t smem;
+    size_t bound;  // what decides whether a call takes this form
 };
 
+constexpr size_t kSmemTwo = 115712;  // shared memory per CTA with two CTAs on an SM
+
 // Shared memory: tables A (hi, lo) over npad dates; a region holding tables B
-// (only with more than 16 basis sums) and two A buffers, later the MOSUM ring;
-// four coefficient planes; the Y stages (TMA loader); barriers.
-MmaLayout mma_layout(int npad, int nhpad, int k, int ring, int elt, bool tma) {
+// (only with more than 16 basis sums), two A buffers, the valid bytes and the pair
+// exchange floats, later the MOSUM ring; the Y stages; barriers.  Y has 3 (float)
+// or 6 (int16) stages, or as few as 2 (float) or 4 (int16) where that lets two CTAs
+// share an SM.  On 1.95 Mi int16 pixels of 586 dates (history 347, ring of 103 slots, 116 KB
+// with six stages and 112 with five) two CTAs took 5.03 ms, one 8.50; with the chunk and
+// group hand-offs per warp and the ring slots counted along, 4.85.
+MmaLayout mma_layout(int npad, int nhpad, int k, int ring, int elt) {
     MmaLayout L{};
     const size_t ta = (size_t)(npad / 8) * kTabLbo;
     const size_t tb = 3 + 6 * k > 16 ? (size_t)(nhpad / 8) * kTabLbo : 0;
-    size_t region = 2 * tb + 2 * (size_t)kBufBytes;
+    const size_t hist = 2 * tb + 2 * (size_t)kBufBytes;
     const size_t rb = (size_t)ring * kTile * 4 + 2 * kTile * 4;  // ring and mailbox
-    if (rb > region) region = rb;
-    region = (region + 1023) & ~(size_t)1023;
-    L.region_bytes = (int)region;
-    L.stages = tma ? (elt == 4 ? 3 : 6) : 0;
     // valid bytes (2 per history block and pixel) and the pair exchange floats
     const int nbh = (nhpad + kBlk - 1) / kBlk;
     const size_t vb = (size_t)nbh * 2 * kTile + 2 * kTile * 4;
-    L.vb_extra = vb <= 2 * (size_t)kCoefPlane ? 0 : (int)((vb + 127) & ~(size_t)127);
-    L.smem = kHdr + 2 * ta + region + 4 * (size_t)kCoefPlane + (size_t)L.stages * kBlk * kTile * elt + L.vb_extra +
-             256;
+    auto up = [](size_t x) { return (x + 1023) & ~(size_t)1023; };
+    const size_t region = up(std::max(hist + vb, rb));
+    const size_t stage = (size_t)kBlk * kTile * elt;
+    L.region_bytes = (int)region;
+    L.stages = elt == 4 ? 3 : 6;
+    const size_t rest = kHdr + 2 * ta + region + 320;
+    for (int s = L.stages; s >= (elt == 4 ? 2 : 4); --s)
+        if (rest + (size_t)s * stage <= kSmemTwo) {
+            L.stages = s;
+            break;
+        }
+    L.smem = rest + (size_t)L.stages * stage;
+    // four 4 KB coefficient planes in shared memory, the valid bytes in two of them or
+    // after 3 or 6 stages: never less than the layout above
+    L.bound = kHdr + 2 * ta + up(std::max(hist, rb)) + 16384 + (size_t)(elt == 4 ? 3 : 6) * stage +
+              (vb <= 8192 ? 0 : (vb + 127) & ~(size_t)127) + 256;
     return L;
 }
 
@@ -902,9 +967,9 @@ bool mma_supported(const bfm_design_s* d, int dtype, int n_hist, double h_frac, 
     if ((dtype != BFM_I16 && dtype != BFM_F32) || !d->d_phi_tc) return false;
     if (!mma_layout_ok(Y, dtype, m)) return false;
     const MmaLayout L = mma_layout(d->npad_tc, (n_hist + 31) / 32 * 32, d->k, ring_len(n_hist, h_frac),
-                                   dtype == BFM_F32 ? 4 : 2, true);
+                                   dtype == BFM_F32 ? 4 : 2);
     if (smem_out) *smem_out = L.smem;
-    return L.smem <= 227 * 1024;
+    return L.bound <= 227 * 1024;
 }
 
 namespace {
@@ -959,10 +1024,9 @@ bool mma_prepare(const bfm_design_s* d, int dtype, const void* Y, const uint32_t
         set_error("tensor-core form: cuTensorMapEncodeTiled failed for Y");
         return false;
     }
-    const MmaLayout L = mma_layout(P.npad, P.nhpad, d->k, P.ring, elt, true);
+    const MmaLayout L = mma_layout(P.npad, P.nhpad, d->k, P.ring, elt);
     P.stages = L.stages;
     P.region_bytes = L.region_bytes;
-    P.vb_extra = L.vb_extra;
     // At least 80 KB, so that at most two CTAs (2 x 256 TMEM columns) share an SM.
     *smem_out = L.smem < 80 * 1024 ? 80 * 1024 : L.smem;
     *Pout = P;
