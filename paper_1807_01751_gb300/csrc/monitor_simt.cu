@@ -160,10 +160,31 @@ __device__ __forceinline__ void simt_block(const CUtensorMap* tmap, const Monito
             return;
         }
     } else {
-        const T* Yp = reinterpret_cast<const T*>(P.Y);
-        for (int idx = threadIdx.x; idx < N * 32; idx += kNW * 32) {
-            const int t = idx >> 5, l = idx & 31;
-            tile[idx] = (p0 + l < P.m) ? Yp[(size_t)t * P.m + p0 + l] : Obs<T>::missing();
+        // every element's copy in flight at once (cp.async); 2-byte elements are below its
+        // smallest size and go through registers, eight loads at a time
+        const T* Yp = reinterpret_cast<const T*>(P.Y) + p;
+        if constexpr (sizeof(T) == 4) {
+            for (int t = w; t < N; t += kNW) {
+                if (active)
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(ptx::smem_u32(tile + t * 32 + lane)),
+                                 "l"(Yp + (size_t)t * P.m)
+                                 : "memory");
+                else
+                    tile[t * 32 + lane] = Obs<T>::missing();
+            }
+            asm volatile("cp.async.wait_all;" ::: "memory");
+        } else {
+            for (int t0 = w; t0 < N; t0 += 8 * kNW) {
+                T v[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const int t = t0 + u * kNW;
+                    v[u] = active && t < N ? __ldg(Yp + (size_t)t * P.m) : Obs<T>::missing();
+                }
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    if (t0 + u * kNW < N) tile[(t0 + u * kNW) * 32 + lane] = v[u];
+            }
         }
         __syncthreads();
     }
