@@ -37,6 +37,7 @@
 #include <vector>
 
 #include "bfm_internal.cuh"
+#include "pair.cuh"
 #include "ptx.cuh"
 #include "stage.cuh"
 
@@ -59,6 +60,7 @@ cudaError_t complete_read_clear_errors(cudaStream_t s, unsigned int* bits) {
 namespace {
 
 using namespace stage;
+using namespace pair;
 
 constexpr int kThreads = 256;
 constexpr int kU1 = 16;  // history dates per load batch (16 loads in flight per thread)
@@ -489,6 +491,472 @@ __global__ void __launch_bounds__(kStaged ? kThreads + 32 : kThreads, 2)
     }
 }
 
+// ---- pixel pairs ---------------------------------------------------------------------
+// The same three passes with two pixels per thread, for larger scenes without an
+// explicit mask.  The staged kernel above is bound by issue: 18.1k lane instructions
+// per pixel, of which the multiply-adds are 7k; the rest are the shared-memory reads
+// of the basis rows (two LDS.128 per date and pass), the ring and the loop's own
+// work.  Blackwell's f32x2 instructions do two IEEE FP32 operations each, and one basis
+// read, ring slot and barrier visit serves both pixels of a thread.  Every pixel goes
+// through the operations of the staged kernel in their order, so the results are the
+// same bits.  What is paired changes with what is independent, so that the tables are
+// read as they are: in pass 1 neighbouring coefficients of one pixel (M' row x y), in
+// the residuals two dates of one pixel (the regressors are stored by date pairs), in the
+// window sums the two pixels.  (Tables holding each value twice, pixels paired
+// throughout, kept the shared-memory pipe 71 % busy: 4.93 ms.)
+// A CTA per SM owns 512 pixels.  8.4 Mi float pixels of 414 dates: 5.55 -> 4.36 ms, now
+// with two warps a scheduler issuing on 52 % of its cycles.
+
+constexpr int kPairThreads = 256;                 // consumer threads of a CTA
+constexpr int kPairPx = 2 * kPairThreads;         // pixels of a tile: two TMA boxes per stage
+constexpr int kPairStageBytes = 2 * kStageBytes;  // 8 (float) or 16 (int16) dates
+constexpr int kPairMaxStages = 6;
+constexpr size_t kPairSmem = 232448;              // opt-in dynamic shared memory per block
+
+struct PairLayout {
+    size_t Xh, Xm, B, XW, ring, stages, bars, total;
+    int nstages;  // 0: does not fit
+};
+
+__host__ __device__ inline PairLayout pair_layout(int N, int n, int K, int h) {
+    PairLayout L{};
+    L.Xh = ((size_t)n * K * 4 + 15) & ~(size_t)15;          // M' [n][K] at 0
+    L.Xm = L.Xh + (size_t)((n + 1) / 2) * K * 8;            // regressors by date pairs: history,
+    L.B = L.Xm + (size_t)((N - n + 1) / 2) * K * 8;         // monitoring dates
+    L.XW = L.B + (size_t)(N - n) * 8;
+    L.ring = (L.XW + (size_t)K * 4 + 127) & ~(size_t)127;
+    L.stages = L.ring + (size_t)h * kPairThreads * 8;
+    const size_t tail = 2 * kPairMaxStages * 8 + 16;
+    L.nstages = 0;
+    for (int s = kPairMaxStages; s >= 3; --s)
+        if (L.stages + (size_t)s * kPairStageBytes + tail <= kPairSmem) {
+            L.nstages = s;
+            break;
+        }
+    L.bars = L.stages + (size_t)L.nstages * kPairStageBytes;
+    L.total = L.bars + tail;
+    return L;
+}
+
+// y - x'beta of four date pairs of two pixels, in the order of `residual` (the first
+// regressor is 1).  row(j): the pair's regressors; bd: each coefficient twice; r comes in
+// as y; x1: the trend regressors.
+template <int K, class Row>
+__device__ __forceinline__ void residual_dates(Row row, const f2 (&bd)[2][K], f2 (&r)[2][4], f2 (&x1)[4]) {
+    f2 yhat[2][4];
+#pragma unroll
+    for (int a = 0; a < K; a += 2) {
+        ulonglong2 x[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) x[j] = *reinterpret_cast<const ulonglong2*>(row(j) + a);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) yhat[e][j] = a == 0 ? bd[e][0] : fma2(x[j].x, bd[e][a], yhat[e][j]);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) yhat[e][j] = fma2(x[j].y, bd[e][a + 1], yhat[e][j]);
+        if (a == 0) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) x1[j] = x[j].y;
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) r[e][j] = add2(r[e][j], neg2(yhat[e][j]));
+}
+
+template <int KH, typename T>
+__global__ void __launch_bounds__(kPairThreads + 32, 1)
+    complete_pair_kernel(const __grid_constant__ CUtensorMap tmap, const CompleteParams P) {
+    constexpr int K = 2 + 2 * KH;
+    constexpr int G = kStageBytes / (256 * (int)sizeof(T));  // dates per stage
+    extern __shared__ __align__(128) float sm[];
+    const int n = P.n, N = P.N, h = P.h;
+    const int64_t m = P.m;
+    const PairLayout Lo = pair_layout(N, n, K, h);
+    unsigned char* base = reinterpret_cast<unsigned char*>(sm);
+    const f2* sM = reinterpret_cast<const f2*>(base);     // [n][K / 2]: neighbouring coefficients
+    f2* sXh = reinterpret_cast<f2*>(base + Lo.Xh);        // [pairs][K]: dates 2j, 2j + 1
+    f2* sXm = reinterpret_cast<f2*>(base + Lo.Xm);        // [pairs][K]: dates n + 2j, n + 2j + 1
+    f2* sNB = reinterpret_cast<f2*>(base + Lo.B);    // [N - n]: -lambda^2 log+((t + 1) / n)
+    float* sXW = reinterpret_cast<float*>(base + Lo.XW);
+    f2* ring = reinterpret_cast<f2*>(base + Lo.ring) + threadIdx.x;  // slot s at ring[s * kPairThreads]
+    unsigned char* stages = base + Lo.stages;
+    const int S = Lo.nstages;
+    uint64_t* full = reinterpret_cast<uint64_t*>(base + Lo.bars);
+    uint64_t* empty = full + kPairMaxStages;
+    volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(empty + kPairMaxStages);
+    const int w0 = n - h + 1;
+    for (int i = threadIdx.x; i < n * K; i += blockDim.x) reinterpret_cast<float*>(base)[i] = P.tab[i];
+    const int nph = (n + 1) / 2, npm = (N - n + 1) / 2;  // date pairs; a last odd date is paired with zeros
+    for (int i = threadIdx.x; i < (nph + npm) * K; i += blockDim.x) {
+        const int j = i / K, a = i - j * K;
+        const int t = j < nph ? 2 * j : n + 2 * (j - nph), end = j < nph ? n : N;
+        const float* x = P.tab + (size_t)(n + t) * K + a;
+        sXh[i] = pack2(x[0], t + 1 < end ? x[K] : 0.f);  // sXm follows sXh
+    }
+    for (int i = threadIdx.x; i < N - n; i += blockDim.x) {
+        const double x = (double)(n + 1 + i) / (double)n;
+        const float b = (float)(P.lam2 * (x <= 2.718281828459045235360287 ? 1.0 : log(x)));
+        sNB[i] = pack2(-b, -b);
+    }
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < S; ++s) {
+            ptx::mbar_init(full + s, 1);
+            ptx::mbar_init(empty + s, kPairThreads / 32);
+        }
+        *abort_flag = 0u;
+        ptx::fence_mbar_init();
+    }
+    if (threadIdx.x < K) {
+        float acc = 0.f;
+        for (int t = w0; t < n; ++t) acc += P.tab[(n + t) * K + threadIdx.x];
+        sXW[threadIdx.x] = acc;
+    }
+    __syncthreads();
+
+    const int64_t ntiles = (m + kPairPx - 1) / kPairPx;
+    if (threadIdx.x >= kPairThreads) {  // the producer warp: one lane issues two boxes per stage
+        if (threadIdx.x == kPairThreads) {
+            ptx::prefetch_tmap(&tmap);
+            const uint64_t keep = l2_evict_last(), normal = l2_evict_normal(), drop = l2_evict_first();
+            int slot = 0;
+            uint32_t lap = 0;
+            bool ok = true;
+            auto issue = [&](int px0, int d0, uint64_t pol) -> bool {
+                if (lap && !wait_released(empty + slot, (lap - 1u) & 1u, abort_flag, kWaitNs)) {
+                    *abort_flag = 1u;
+                    atomicOr(&g_bfm_complete_err, 1u);
+                    return false;
+                }
+                if (*abort_flag) return false;
+                ptx::mbar_arrive_expect_tx(full + slot, (uint32_t)kPairStageBytes);  // boxes are always full
+                unsigned char* dst = stages + (size_t)slot * kPairStageBytes;
+                tma_box(dst, &tmap, full + slot, px0, d0, pol);
+                tma_box(dst + kStageBytes, &tmap, full + slot, px0 + 256, d0, pol);
+                if (++slot == S) {
+                    slot = 0;
+                    ++lap;
+                }
+                return true;
+            };
+            for (int64_t tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
+                const int px0 = (int)(tile * kPairPx);
+                for (int d0 = 0; d0 < n && ok; d0 += G) ok = issue(px0, d0, keep);
+                for (int d0 = 0; d0 < n && ok; d0 += G) ok = issue(px0, d0, drop);
+                for (int d0 = n; d0 < N && ok; d0 += G) ok = issue(px0, d0, normal);
+            }
+            // copies still in flight land before the CTA's shared memory is released
+            for (int i = 0; i < S; ++i) {
+                const uint32_t uses = lap + (i < slot ? 1u : 0u);
+                if (uses) ptx::mbar_wait_bounded(full + i, (uses - 1u) & 1u, kWaitNs);
+            }
+        }
+        return;
+    }
+
+    // stage hand-off as in the staged kernel: a warp whose wait gave up is `bad` and
+    // releases nothing from then on
+    bool bad = false;
+    int cslot = 0;
+    uint32_t cphase = 0;
+    // thread t: pixel t of either box
+    const T* const scol = reinterpret_cast<const T*>(stages) + threadIdx.x;
+    auto acquire = [&]() -> const T* {
+        const int slot = cslot;
+        bool ok = ptx::mbar_try_wait(full + slot, cphase);
+        if (!__all_sync(~0u, ok)) {
+            if (!ok) ok = wait_released(full + slot, cphase, abort_flag, kWaitNs);
+            if (__any_sync(~0u, !ok)) {
+                if ((threadIdx.x & 31) == 0 && !bad) {
+                    *abort_flag = 1u;
+                    atomicOr(&g_bfm_complete_err, 1u);
+                }
+                bad = true;
+            }
+        }
+        return scol + (size_t)slot * (kPairStageBytes / sizeof(T));
+    };
+    auto release = [&]() {
+        __syncwarp();
+        if ((threadIdx.x & 31) == 0 && !bad) mbar_arrive(empty + cslot);
+        const int ns = cslot + 1;
+        cphase ^= ns == S ? 1u : 0u;
+        cslot = ns == S ? 0 : ns;
+    };
+    const float qnan = __int_as_float(0x7fc00000);
+    auto write_unfitted = [&](int64_t p, int st) {
+        P.brk[p] = -1;
+        P.mean[p] = qnan;
+        P.sigma[p] = qnan;
+#pragma unroll
+        for (int a = 0; a < K; ++a) P.beta[(size_t)a * m + p] = qnan;
+        P.status[p] = (uint8_t)st;
+        if (P.maxmo) P.maxmo[p] = qnan;
+    };
+
+    int64_t tile = blockIdx.x;
+    for (; tile < ntiles; tile += gridDim.x) {
+        const int64_t p = tile * kPairPx + threadIdx.x;
+        constexpr int kBox = kStageBytes / (int)sizeof(T);  // elements from pixel t to pixel 256 + t
+        // pass 1: beta0 = M y (coefficients in neighbouring pairs), max |y|
+        f2 bp[2][K / 2];
+        float ymax[2] = {0.f, 0.f};
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+#pragma unroll
+            for (int a = 0; a < K / 2; ++a) bp[e][a] = 0ull;
+        auto pass1 = [&](int d0, auto full_c) {
+            constexpr bool full = decltype(full_c)::value;
+            const int cnt = full ? G : n - d0;
+            const T* st = acquire();
+#pragma unroll
+            for (int u = 0; u < G; ++u) {
+                const f2* q = sM + (full ? d0 + u : min(d0 + u, n - 1)) * (K / 2);
+                f2 mt[K / 2];
+                if constexpr (K % 4 == 0) {
+#pragma unroll
+                    for (int a = 0; a < K / 2; a += 2) {
+                        const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(q + a);
+                        mt[a] = v.x;
+                        mt[a + 1] = v.y;
+                    }
+                } else {
+#pragma unroll
+                    for (int a = 0; a < K / 2; ++a) mt[a] = q[a];
+                }
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const float v = (full || u < cnt) ? obs_value(st[u * 256 + e * kBox]) : 0.f;
+                    ymax[e] = fmaxf(ymax[e], fabsf(v));
+                    const f2 vv = pack2(v, v);
+#pragma unroll
+                    for (int a = 0; a < K / 2; ++a) bp[e][a] = fma2(mt[a], vv, bp[e][a]);
+                }
+            }
+            release();
+        };
+        int d0 = 0;
+        for (; d0 + G <= n && !bad; d0 += G) pass1(d0, std::true_type{});
+        if (d0 < n && !bad) pass1(d0, std::false_type{});
+        f2 bd[2][K];  // each coefficient twice
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+#pragma unroll
+            for (int a = 0; a < K; ++a) {
+                const float v = half2(bp[e][a / 2], a & 1);
+                bd[e][a] = pack2(v, v);
+            }
+
+        // eight dates from u0 of a stage, by date pairs
+        auto load_pairs = [&](const T* st, int u0, int cnt, bool full, f2 (&r)[2][4]) {
+#pragma unroll
+            for (int e = 0; e < 2; ++e)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int u = u0 + 2 * j;
+                    const T* q = st + u * 256 + e * kBox;
+                    r[e][j] = pack2(full || u < cnt ? obs_value(q[0]) : 0.f, full || u + 1 < cnt ? obs_value(q[256]) : 0.f);
+                }
+        };
+        // pass 2: history residuals, sum of squares, refinement of intercept and trend, first window
+        f2 c01[2] = {0ull, 0ull}, W0 = 0ull;
+        float ss[2] = {0.f, 0.f};
+        auto pass2 = [&](int d0, auto full_c, auto win_c) {
+            constexpr bool full = decltype(full_c)::value;
+            constexpr bool win = decltype(win_c)::value;  // the batch may reach the first window (t >= w0)
+            const int cnt = full ? G : n - d0;
+            const T* st = acquire();
+#pragma unroll
+            for (int u0 = 0; u0 < G; u0 += 8) {
+                f2 r[2][4], x1[4];
+                load_pairs(st, u0, cnt, full, r);
+                const int j0 = (d0 + u0) / 2;
+                residual_dates<K>([&](int j) { return sXh + (full ? j0 + j : min(j0 + j, nph - 1)) * K; }, bd, r, x1);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int u = u0 + i, t = d0 + u;
+                    const f2 m01 = sM[(full ? t : min(t, n - 1)) * (K / 2)];
+                    float re[2];
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        re[e] = half2(r[e][i / 2], i & 1);
+                        if (!full) re[e] = u < cnt ? re[e] : 0.f;
+                        ss[e] = fmaf(re[e], re[e], ss[e]);
+                        c01[e] = fma2(m01, pack2(re[e], re[e]), c01[e]);
+                    }
+                    if (win && t >= w0 && (full || u < cnt)) {
+                        const f2 rp = pack2(re[0], re[1]);
+                        W0 = add2(W0, rp);
+                        ring[(t - w0) * kPairThreads] = rp;
+                    }
+                }
+            }
+            release();
+        };
+        for (d0 = 0; d0 + G <= n && !bad; d0 += G) {
+            if (d0 + G <= w0)
+                pass2(d0, std::true_type{}, std::false_type{});
+            else
+                pass2(d0, std::true_type{}, std::true_type{});
+        }
+        if (d0 < n && !bad) pass2(d0, std::false_type{}, std::true_type{});
+        // residuals from here on: beta0 with the intercept and trend corrected by (c0, c1)
+        f2 W, c0d[2], c1d[2];
+        float sig[2], inv_scale[2];
+        bool degenerate[2];
+        {
+            float w[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const float c0 = half2(c01[e], 0), c1 = half2(c01[e], 1);
+                w[e] = half2(W0, e) - fmaf(sXW[1], c1, sXW[0] * c0);
+                c0d[e] = pack2(c0, c0);
+                c1d[e] = pack2(c1, c1);
+                sig[e] = sqrtf(ss[e] / (float)(n - K));
+                degenerate[e] = !(sig[e] > 1e-6f * ymax[e]) || ymax[e] == 0.f;
+                inv_scale[e] = degenerate[e] ? 0.f : 1.f / (sig[e] * sqrtf((float)n));
+            }
+            W = pack2(w[0], w[1]);
+            const f2 c0 = pack2(half2(c0d[0], 0), half2(c0d[1], 0)), c1 = pack2(half2(c1d[0], 0), half2(c1d[1], 0));
+            const float* xh = reinterpret_cast<const float*>(sXh);
+            for (int d = w0; d < n; ++d) {
+                const float x = xh[((d >> 1) * K + 1) * 2 + (d & 1)];
+                f2* q = ring + (d - w0) * kPairThreads;
+                *q = add2(*q, neg2(fma2(pack2(x, x), c1, c0)));
+            }
+        }
+        const f2 inv2 = pack2(inv_scale[0] * inv_scale[0], inv_scale[1] * inv_scale[1]);
+
+        // pass 3: monitoring dates
+        int brk[2] = {-1, -1};
+        float sh[2] = {0.f, 0.f}, sl[2] = {0.f, 0.f};
+        float wmax[2] = {-INFINITY, -INFINITY}, wmin[2] = {INFINITY, INFINITY};
+        int slot = h - 1;  // ring slot of date t: (t - w0) mod h
+        auto pass3 = [&](int d0, auto full_c, auto ext_c) {
+            constexpr bool full = decltype(full_c)::value;
+            constexpr bool ext = decltype(ext_c)::value;  // the largest |MO| is wanted
+            const int cnt = full ? G : N - d0;
+            const T* st = acquire();
+            f2 blk = 0ull, wv[G];
+            float cmax[2] = {-INFINITY, -INFINITY};
+#pragma unroll
+            for (int u0 = 0; u0 < G; u0 += 8) {
+                f2 r[2][4], x1[4];
+                load_pairs(st, u0, cnt, full, r);
+                const int j0 = (d0 - n + u0) / 2;
+                residual_dates<K>([&](int j) { return sXm + (full ? j0 + j : min(j0 + j, npm - 1)) * K; }, bd, r, x1);
+#pragma unroll
+                for (int e = 0; e < 2; ++e)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) r[e][j] = add2(r[e][j], neg2(fma2(x1[j], c1d[e], c0d[e])));
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int u = u0 + i, t = d0 + u;
+                    wv[u] = 0ull;
+                    if (full || u < cnt) {
+                        const f2 rp = pack2(half2(r[0][i / 2], i & 1), half2(r[1][i / 2], i & 1));
+                        f2* q = ring + slot * kPairThreads;
+                        const f2 ro = t > n ? *q : 0ull;
+                        *q = rp;
+                        slot = slot + 1 == h ? 0 : slot + 1;
+                        W = add2(add2(W, rp), neg2(ro));
+                        wv[u] = W;
+                        float k0, k1;
+                        unpack2(fma2(mul2(W, W), inv2, sNB[t - n]), k0, k1);
+                        cmax[0] = fmaxf(cmax[0], k0);
+                        cmax[1] = fmaxf(cmax[1], k1);
+                        blk = add2(blk, W);
+                        if (ext) {
+                            unpack2(W, k0, k1);
+                            wmax[0] = fmaxf(wmax[0], k0);
+                            wmax[1] = fmaxf(wmax[1], k1);
+                            wmin[0] = fminf(wmin[0], k0);
+                            wmin[1] = fminf(wmin[1], k1);
+                        }
+                    }
+                }
+            }
+            if ((brk[0] < 0 && cmax[0] > 0.f) || (brk[1] < 0 && cmax[1] > 0.f)) {
+#pragma unroll
+                for (int u = 0; u < G; ++u)
+                    if (full || u < cnt) {
+                        float k0, k1;
+                        unpack2(fma2(mul2(wv[u], wv[u]), inv2, sNB[d0 + u - n]), k0, k1);
+                        if (brk[0] < 0 && k0 > 0.f) brk[0] = d0 + u;
+                        if (brk[1] < 0 && k1 > 0.f) brk[1] = d0 + u;
+                    }
+            }
+            float k0, k1;
+            unpack2(blk, k0, k1);
+            comp_add(sh[0], sl[0], k0);
+            comp_add(sh[1], sl[1], k1);
+            release();
+        };
+        d0 = n;
+        if (P.maxmo) {
+            for (; d0 + G <= N && !bad; d0 += G) pass3(d0, std::true_type{}, std::true_type{});
+            if (d0 < N && !bad) pass3(d0, std::false_type{}, std::true_type{});
+        } else {
+            for (; d0 + G <= N && !bad; d0 += G) pass3(d0, std::true_type{}, std::false_type{});
+            if (d0 < N && !bad) pass3(d0, std::false_type{}, std::false_type{});
+        }
+        if (bad) break;
+
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            float bl[K];
+#pragma unroll
+            for (int a = 0; a < K; ++a) bl[a] = half2(bd[e][a], 0);
+            const int64_t pe = p + 256 * e;
+            if (pe >= m) continue;
+            if (isnan(bl[0]) || isnan(sh[e])) {  // a missing value met in the history or the monitoring period
+                write_unfitted(pe, BFM_PX_INCOMPLETE);
+                continue;
+            }
+            P.brk[pe] = degenerate[e] ? -1 : brk[e];
+            P.mean[pe] = degenerate[e] ? 0.f : (sh[e] + sl[e]) * inv_scale[e] / (float)(N - n);
+            P.sigma[pe] = sig[e];
+            // beta of the centred trend -> raw parameterisation of Eq. 2
+            const float beta0 = bl[0] + half2(c0d[e], 0), beta1 = bl[1] + half2(c1d[e], 0);
+            P.beta[pe] = fmaf(-beta1, P.c_over_s, beta0);
+            P.beta[(size_t)m + pe] = beta1 * P.inv_s;
+#pragma unroll
+            for (int a = 2; a < K; ++a) P.beta[(size_t)a * m + pe] = bl[a];
+            P.status[pe] = degenerate[e] ? BFM_PX_DEGENERATE : BFM_PX_OK;
+            // largest |MO| (positive on an exact tie of opposite signs)
+            if (P.maxmo)
+                P.maxmo[pe] = degenerate[e] ? 0.f : (wmax[e] >= -wmin[e] ? wmax[e] : wmin[e]) * inv_scale[e];
+        }
+    }
+    if (bad) {
+        // a stage wait gave up: mark this thread's unfinished pixels
+        if ((threadIdx.x & 31) == 0) {
+            *abort_flag = 1u;
+            atomicOr(&g_bfm_complete_err, 1u);
+        }
+        for (; tile < ntiles; tile += gridDim.x)
+            for (int e = 0; e < 2; ++e) {
+                const int64_t p = tile * kPairPx + threadIdx.x + 256 * e;
+                if (p < m) write_unfitted(p, BFM_PX_TIMEOUT);
+            }
+    }
+}
+
+template <int KH, typename T>
+bfm_status launch_pair(const CUtensorMap& tm, const CompleteParams& P, int grid, size_t smem, cudaStream_t st) {
+    auto* fn = complete_pair_kernel<KH, T>;
+    const cudaError_t ea = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmem);
+    if (ea != cudaSuccess) return cuda_fail(ea, "bfm_monitor (complete): shared memory attribute");
+    fn<<<grid, kPairThreads + 32, smem, st>>>(tm, P);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return cuda_fail(e, "bfm_monitor (complete): launch");
+    return BFM_OK;
+}
+
 template <int KH, typename T, bool kMask, bool kStaged>
 bfm_status launch_variant(const CUtensorMap& tm, const CompleteParams& P, int grid, size_t smem, cudaStream_t st) {
     auto* fn = complete_kernel<KH, T, kMask, kStaged>;
@@ -656,6 +1124,23 @@ bfm_status launch_complete(bfm_design_s* d, int dtype, const void* Y, const uint
                             const_cast<void*>(Y), gdim, gstride, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
                             CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    }
+    if (staged && !P.mask && shared == BFM_PX_OK) {
+        // pixel pairs: scenes of at least a tile of 512 pixels per SM (smaller ones leave SMs to
+        // the other kernel's two CTAs of 256) whose tables, ring and three stages fit, with
+        // the history of the resident pixels within the L2 budget
+        const PairLayout pl = pair_layout(d->N, n_hist, d->K, P.h);
+        const int64_t ptiles = (m + kPairPx - 1) / kPairPx;
+        if (pl.nstages && ptiles >= (int64_t)sms && (double)kPairPx * n_hist * (double)elt * sms <= kL2Budget) {
+            const int pgrid = (int)(ptiles < sms ? ptiles : sms);
+            if (dtype == BFM_F32)
+                return d->k == 1   ? launch_pair<1, float>(tm, P, pgrid, pl.total, stream)
+                       : d->k == 2 ? launch_pair<2, float>(tm, P, pgrid, pl.total, stream)
+                                   : launch_pair<3, float>(tm, P, pgrid, pl.total, stream);
+            return d->k == 1   ? launch_pair<1, int16_t>(tm, P, pgrid, pl.total, stream)
+                   : d->k == 2 ? launch_pair<2, int16_t>(tm, P, pgrid, pl.total, stream)
+                               : launch_pair<3, int16_t>(tm, P, pgrid, pl.total, stream);
+        }
     }
     const size_t smem = complete_smem_bytes(d->N, n_hist, d->K, P.h, staged);
     if (staged) {
