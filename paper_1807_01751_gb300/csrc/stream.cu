@@ -17,7 +17,8 @@
 //       residuals s1 = s0 - delta'c (Algorithm 1 step 5), sigma-hat, h_p.
 //   B   residuals of the first window's h_p - 1 valid history observations
 //       (valid ranks n_p - h_p + 1 .. n_p - 1, 0-based) into a per-thread
-//       ring in shared memory, and their sum.
+//       ring in shared memory, and their sum; from the earliest date at which
+//       a window of the CTA starts (found in A').
 //   C   at each valid monitoring observation (position J = n_p + 1 ..): the
 //       window sum gains its residual and loses the ring slot it replaces
 //       (the observation h_p positions earlier); MO_J = W / (sigma-hat
@@ -26,6 +27,12 @@
 // Residuals in B and C hold the intercept and trend coefficients as beta0 +
 // delta (hi + lo): a float rounding of those two would enter all h_p
 // residuals of a window alike.
+//
+// Bound by instruction issue (75 % of the cycles).  Pass B from the window's start
+// instead of the history's, and the boundary only where a batch's largest |MO| can
+// reach it, took 500k int16 pixels of 522 dates (one harmonic) from 661 to 548 us.  Two
+// pixels per thread with f32x2 arithmetic issued a third fewer instructions, but the
+// ring leaves room for 512 pixels, so eight warps: 52 % issue, 627 us; not kept.
 #include <cudaTypedefs.h>
 
 #include <atomic>
@@ -122,9 +129,12 @@ __host__ __device__ inline Layout stream_layout(int N, int n, int K, int NB, int
     L.ring = L.xm + up128(sizeof(float) * (size_t)(N - n) * K);
     L.stages = L.ring + up128(sizeof(float) * (size_t)hmax * kThreads);
     L.bars = L.stages + (size_t)kStageArea;
-    L.total = L.bars + 2 * kMaxStages * sizeof(uint64_t) + 16;
+    L.total = L.bars + 2 * kMaxStages * sizeof(uint64_t) + 16;  // what decides whether a call takes this form
     return L;
 }
+
+// Barriers (with the one of the window starts), the abort flag and the window starts.
+constexpr size_t kBarBytes = 2 * kMaxStages * sizeof(uint64_t) + 32;
 
 template <int KH, typename T, bool kMask>
 __global__ void __launch_bounds__(kThreads + 32, 2)
@@ -145,6 +155,8 @@ __global__ void __launch_bounds__(kThreads + 32, 2)
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + Lo.bars);
     uint64_t* empty = full + kMaxStages;
     volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(empty + kMaxStages);
+    uint64_t* dminb = empty + kMaxStages + 1;  // every warp's earliest window start published
+    volatile unsigned char* s_dmin = smem + Lo.bars + kBarBytes - 16;  // [2][8] start / 8, by tile parity and warp
     for (int i = threadIdx.x; i < n * NB; i += blockDim.x) sPhi[i] = P.basis[i];
     for (int i = threadIdx.x; i < (N - n) * K; i += blockDim.x) {
         const int r = i / K;
@@ -155,47 +167,64 @@ __global__ void __launch_bounds__(kThreads + 32, 2)
             ptx::mbar_init(full + s, 1);
             ptx::mbar_init(empty + s, kThreads / 32);
         }
+        ptx::mbar_init(dminb, kThreads / 32);
         *abort_flag = 0u;
         ptx::fence_mbar_init();
     }
     __syncthreads();
+    // the date pass B starts at: the CTA's earliest window start, a multiple of G
+    auto start_b = [&](uint32_t par) -> int {
+        int d = s_dmin[8 * par];
+#pragma unroll
+        for (int w = 1; w < kThreads / 32; ++w) d = min(d, (int)s_dmin[8 * par + w]);
+        return d * 8;
+    };
 
-    // stage sequence of one tile: passes A, A', B over the history (ng1
-    // boxes each), pass C over the monitoring dates (ng3 boxes); stage j of
-    // this CTA is box j % Q of its tile j / Q, in slot j % kStages
     const int64_t ntiles = (m + kThreads - 1) / kThreads;
-    const int ng1 = (n + G - 1) / G, ng3 = (N - n + G - 1) / G, Q = 3 * ng1 + ng3;
-    const int64_t my_tiles = (int64_t)blockIdx.x < ntiles ? (ntiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
-    const int64_t total = my_tiles * Q;
-
     if (threadIdx.x >= kThreads) {  // the producer warp: one lane issues the boxes
         if (threadIdx.x == kThreads) {
             ptx::prefetch_tmap(&tmap);
             const uint64_t keep = l2_evict_last(), normal = l2_evict_normal(), drop = l2_evict_first();
-            int64_t js = 0;
-            for (; js < total; ++js) {
-                const int slot = (int)(js % kStages);
+            int slot = 0;
+            uint32_t lap = 0, dpar = 0;  // laps of the ring completed; the tile's parity
+            bool ok = true;
+            auto fail = [&]() -> bool {
+                *abort_flag = 1u;
+                atomicOr(&g_bfm_stream_err, 1u);
+                return false;
+            };
+            auto issue = [&](int px0, int d0, uint64_t pol) -> bool {
                 // the slot's previous stage released by every consumer warp
-                if (js >= kStages &&
-                    !wait_released(empty + slot, (uint32_t)(((js / kStages) - 1) & 1), abort_flag, kWaitNs)) {
-                    *abort_flag = 1u;
-                    atomicOr(&g_bfm_stream_err, 1u);
-                    break;
-                }
-                if (*abort_flag) break;
-                const int64_t tl = js / Q;
-                const int k = (int)(js - tl * Q);
-                const int px0 = (int)((blockIdx.x + tl * gridDim.x) * kThreads);
-                const int d0 = k < 3 * ng1 ? (k % ng1) * G : n + (k - 3 * ng1) * G;
-                // passes A and A' keep the history in L2 for the next history
-                // pass; pass B is its last use
-                const uint64_t pol = k < 2 * ng1 ? keep : (k < 3 * ng1 ? drop : normal);
+                if (lap && !wait_released(empty + slot, (lap - 1u) & 1u, abort_flag, kWaitNs)) return fail();
+                if (*abort_flag) return false;
                 ptx::mbar_arrive_expect_tx(full + slot, (uint32_t)kStageBytes);  // boxes are always full
                 tma_box(stages + slot * kStageBytes, &tmap, full + slot, px0, d0, pol);
+                if (++slot == kStages) {
+                    slot = 0;
+                    ++lap;
+                }
+                return true;
+            };
+            for (int64_t tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
+                const int px0 = (int)(tile * kThreads);
+                // passes A and A' keep the history in L2 for the next history
+                // pass; pass B, from the earliest window start on, is its last use
+                for (int d0 = 0; d0 < n && ok; d0 += G) ok = issue(px0, d0, keep);
+                for (int d0 = 0; d0 < n && ok; d0 += G) ok = issue(px0, d0, keep);
+                if (!ok) break;
+                if (!wait_released(dminb, dpar, abort_flag, kWaitNs)) {
+                    fail();
+                    break;
+                }
+                for (int d0 = start_b(dpar); d0 < n && ok; d0 += G) ok = issue(px0, d0, drop);
+                dpar ^= 1u;
+                for (int d0 = n; d0 < N && ok; d0 += G) ok = issue(px0, d0, normal);
             }
             // copies still in flight land before the CTA's shared memory is released
-            for (int64_t i = js > kStages ? js - kStages : 0; i < js; ++i)
-                ptx::mbar_wait_bounded(full + (i % kStages), (uint32_t)((i / kStages) & 1), kWaitNs);
+            for (int i = 0; i < kStages; ++i) {
+                const uint32_t uses = lap + (i < slot ? 1u : 0u);
+                if (uses) ptx::mbar_wait_bounded(full + i, (uses - 1u) & 1u, kWaitNs);
+            }
         }
         return;
     }
@@ -214,12 +243,12 @@ __global__ void __launch_bounds__(kThreads + 32, 2)
     // matter (its pixels end as TIMEOUT), but it releases none, so the producer
     // never refills a slot whose copy may still be in flight.
     const bool test_mode = P.wait_ns < 1000u;
-    auto acquire = [&]() -> const T* {
-        const int slot = cslot;
-        bool ok = !test_mode && ptx::mbar_try_wait(full + slot, cphase);
+    uint32_t dpar = 0;
+    auto wait_w = [&](uint64_t* bar, uint32_t parity) {
+        bool ok = !test_mode && ptx::mbar_try_wait(bar, parity);
         if (!__all_sync(~0u, ok)) {
-            if (!ok) ok = test_mode ? ptx::mbar_test_wait(full + slot, cphase)
-                                    : wait_released(full + slot, cphase, abort_flag, P.wait_ns);
+            if (!ok)
+                ok = test_mode ? ptx::mbar_test_wait(bar, parity) : wait_released(bar, parity, abort_flag, P.wait_ns);
             if (__any_sync(~0u, !ok)) {
                 if ((threadIdx.x & 31) == 0 && !bad) {
                     *abort_flag = 1u;
@@ -228,7 +257,10 @@ __global__ void __launch_bounds__(kThreads + 32, 2)
                 bad = true;
             }
         }
-        return reinterpret_cast<const T*>(stages + slot * kStageBytes) + threadIdx.x;
+    };
+    auto acquire = [&]() -> const T* {
+        wait_w(full + cslot, cphase);
+        return reinterpret_cast<const T*>(stages + cslot * kStageBytes) + threadIdx.x;
     };
     auto release = [&]() {  // this warp is done with stage j
         __syncwarp();
@@ -253,16 +285,22 @@ __global__ void __launch_bounds__(kThreads + 32, 2)
     for (; tile < ntiles; tile += gridDim.x) {
         const int64_t p = tile * kThreads + threadIdx.x;
         const bool active = p < m;
-        const uint32_t* mp = kMask ? P.mask + (active ? (p >> 5) : 0) : nullptr;
-        const uint32_t mbit = 1u << (p & 31);
-        const size_t mws = (size_t)P.mask_words;
-        // observation u of a stage whose dates start at d0: value (0 when
+        const int64_t wcol = p >> 5;  // the warp's 32 pixels share one mask word per date
+        MaskBits mb{kMask ? P.mask + wcol : nullptr, (size_t)P.mask_words, kMask && wcol < P.mask_words ? N : 0};
+        const int lane = threadIdx.x & 31;
+        // the mask bits of the batch of dates at d0, of a pass that starts at base
+        auto mask_bits = [&](int d0, int base) -> uint32_t {
+            if (!kMask) return 0u;
+            if (((d0 - base) & 31) == 0) mb.next(d0, lane);
+            return mb.cur >> ((d0 - base) & 31);
+        };
+        // observation u of a stage with these mask bits: value (0 when
         // missing) and 1/0 for valid/missing; in a partial batch (full =
         // false) the dates from cnt on do not belong to the pass
-        auto get = [&](const T* st, int d0, int u, int cnt, bool full, float& y) -> float {
+        auto get = [&](const T* st, uint32_t bits, int u, int cnt, bool full, float& y) -> float {
             bool ok = obs(st[u * kThreads], y);
             if (!full) ok = ok && u < cnt;
-            if (kMask) ok = ok && (mp[(size_t)(d0 + u) * mws] & mbit);
+            if (kMask) ok = ok && ((bits >> u) & 1u);
             y = ok ? y : 0.f;
             return ok ? 1.f : 0.f;
         };
@@ -278,10 +316,11 @@ __global__ void __launch_bounds__(kThreads + 32, 2)
             constexpr bool full = decltype(full_c)::value;
             const int cnt = full ? G : n - d0;
             const T* st = acquire();
+            const uint32_t bits = mask_bits(d0, 0);
 #pragma unroll
             for (int u = 0; u < G; ++u) {
                 float y;
-                const float v = get(st, d0, u, cnt, full, y);
+                const float v = get(st, bits, u, cnt, full, y);
                 const float* ph = sPhi + (full ? d0 + u : min(d0 + u, n - 1)) * NB;
 #pragma unroll
                 for (int i = 0; i < NBR; ++i) S[i] = fmaf(ph[i], v, S[i]);
@@ -292,9 +331,12 @@ __global__ void __launch_bounds__(kThreads + 32, 2)
             release();
         };
         int d0 = 0;
+        if (kMask) mb.open(0, lane);
         for (; d0 + G <= n && !bad; d0 += G) passA(d0, std::true_type{});
         if (d0 < n && !bad) passA(d0, std::false_type{});
         const int np = (int)S[0];  // basis row 0 is 1: S[0] counts the valid history dates
+        int hp = (int)floor(P.h_frac * (double)np);
+        hp = hp < 1 ? 1 : (hp > np ? np : hp);
         float b0[K];
         bool nonsingular;
         {
@@ -304,29 +346,51 @@ __global__ void __launch_bounds__(kThreads + 32, 2)
             chol_solve<K>(Lc, dinv, Bv, b0);
         }
 
-        // pass A': residuals r0 of the first solution, refinement sums c = X'M r0
+        const bool fit = np > K && nonsingular;
+
+        // pass A': residuals r0 of the first solution, refinement sums c = X'M r0, and the
+        // date of the window's oldest history observation (0-based valid rank n_p - h_p + 1)
+        int rem = fit ? np - hp + 1 : np, wdate = n;
         float cr[K];
 #pragma unroll
         for (int a = 0; a < K; ++a) cr[a] = 0.f;
         float ss0 = 0.f;
-        auto passA2 = [&](int d0, auto full_c) {
+        auto passA2 = [&](int d0, auto full_c, auto scan_c, const T* st, uint32_t bits) {
             constexpr bool full = decltype(full_c)::value;
+            constexpr bool scan = decltype(scan_c)::value;  // a pixel of the warp may reach its window
             const int cnt = full ? G : n - d0;
-            const T* st = acquire();
 #pragma unroll
             for (int u = 0; u < G; ++u) {
                 float y;
-                const float v = get(st, d0, u, cnt, full, y);
+                const float v = get(st, bits, u, cnt, full, y);
                 const float* ph = sPhi + (full ? d0 + u : min(d0 + u, n - 1)) * NB;
                 const float r = residual<K>(y, ph, b0) * v;
                 ss0 = fmaf(r, r, ss0);
 #pragma unroll
                 for (int a = 0; a < K; ++a) cr[a] = fmaf(ph[a], r, cr[a]);
+                if (scan) wdate = v != 0.f && rem == 0 ? d0 + u : wdate;
+                rem -= v != 0.f ? 1 : 0;
             }
-            release();
         };
-        for (d0 = 0; d0 + G <= n && !bad; d0 += G) passA2(d0, std::true_type{});
-        if (d0 < n && !bad) passA2(d0, std::false_type{});
+        if (kMask) mb.open(0, lane);
+        for (d0 = 0; d0 < n && !bad; d0 += G) {
+            const T* st = acquire();
+            const uint32_t bits = mask_bits(d0, 0);
+            if (d0 + G > n)
+                passA2(d0, std::false_type{}, std::true_type{}, st, bits);
+            else if (__any_sync(~0u, rem < G))
+                passA2(d0, std::true_type{}, std::true_type{}, st, bits);
+            else
+                passA2(d0, std::true_type{}, std::false_type{}, st, bits);
+            release();
+        }
+        {
+            const unsigned w = __reduce_min_sync(~0u, (unsigned)(active ? wdate : n));
+            if ((threadIdx.x & 31) == 0) {
+                s_dmin[8 * dpar + (threadIdx.x >> 5)] = (unsigned char)(w >> 3);  // n / 8 <= 224
+                mbar_arrive(dminb);
+            }
+        }
         float dl[K];
         {
             float Gm[K][K], Lc[K][K], dinv[K];
@@ -337,11 +401,8 @@ __global__ void __launch_bounds__(kThreads + 32, 2)
         float dc = 0.f;
 #pragma unroll
         for (int a = 0; a < K; ++a) dc = fmaf(dl[a], cr[a], dc);
-        const bool fit = np > K && nonsingular;
         const float sig = sqrtf(fmaxf(ss0 - dc, 0.f) / (float)(np - K));
         const bool degenerate = !(sig > kDegenerateRatio * ymax) || ymax == 0.f;
-        int hp = (int)floor(P.h_frac * (double)np);
-        hp = hp < 1 ? 1 : (hp > np ? np : hp);
         if (!fit) hp = 1;  // keeps the ring arithmetic in range; nothing of it is used
         float bres[K];  // coefficients of the residuals: intercept and trend as hi (bres) + lo (dl)
 #pragma unroll
@@ -352,84 +413,101 @@ __global__ void __launch_bounds__(kThreads + 32, 2)
         const float lam2ln2 = P.lam2 * kLn2f, blg = lam2ln2 * log2f((float)np);
         const float jlimf = (float)floor(kEuler * (double)np);  // J / n_p <= e  <=>  J <= jlim
 
+        wait_w(dminb, dpar);
+        if (bad) break;
+        const int db = start_b(dpar);
+        dpar ^= 1u;
+
         // pass B: the first window's h_p - 1 valid history residuals into the
-        // ring (valid ranks wq .. n_p - 1 -> slots 0 .. h_p - 2), branch-free
-        const int wq = fit ? np - hp + 1 : np;  // 0-based valid rank of the window's oldest history observation
+        // ring, from the CTA's earliest window start, branch-free
         float W = 0.f;
-        int q = -wq;  // valid rank minus wq: the slot of the next valid observation when >= 0
-        auto passB = [&](int d0, auto full_c) {
-            constexpr bool full = decltype(full_c)::value;
-            const int cnt = full ? G : n - d0;
+        int slot = 0;  // ring slot of the next observation
+        if (kMask) mb.open(db, lane);
+        for (d0 = db; d0 < n && !bad; d0 += G) {
             const T* st = acquire();
-            if (__any_sync(~0u, q + G > 0)) {  // some pixel of the warp may reach its window in this batch
+            const uint32_t bits = mask_bits(d0, db);
+            if (__any_sync(~0u, wdate < d0 + G)) {
 #pragma unroll
                 for (int u = 0; u < G; ++u) {
                     float y;
-                    const float v = get(st, d0, u, cnt, full, y);
-                    const float r =
-                        residual2<K>(y, sPhi + (full ? d0 + u : min(d0 + u, n - 1)) * NB, bres, lo0, lo1);
-                    const bool take = v != 0.f && q >= 0;
-                    if (take) ring[q * kThreads] = r;
+                    const float v = get(st, bits, u, n - d0, false, y);
+                    const float r = residual2<K>(y, sPhi + min(d0 + u, n - 1) * NB, bres, lo0, lo1);
+                    const bool take = v != 0.f && d0 + u >= wdate;
+                    if (take) ring[slot * kThreads] = r;
                     W += take ? r : 0.f;
-                    q += v != 0.f ? 1 : 0;
-                }
-            } else {  // only count the valid observations
-#pragma unroll
-                for (int u = 0; u < G; ++u) {
-                    float y;
-                    q += get(st, d0, u, cnt, full, y) != 0.f ? 1 : 0;
+                    slot += take ? 1 : 0;
                 }
             }
             release();
-        };
-        for (d0 = 0; d0 + G <= n && !bad; d0 += G) passB(d0, std::true_type{});
-        if (d0 < n && !bad) passB(d0, std::false_type{});
+        }
 
         // pass C: the monitoring observations, branch-free per date
         float Jf = (float)(np + 1);  // position of the next valid monitoring observation (exact in float)
-        int slot = hp - 1;  // ring slot of the next observation
+        slot = hp - 1;
+        ring[slot * kThreads] = 0.f;  // the first monitoring step finds h_p - 1 residuals
         int brk = -1;
         float sh = 0.f, sl = 0.f, wmax = -INFINITY, wmin = INFINITY;
-        auto passC = [&](int d0, auto full_c) {
+        auto passC = [&](int d0, auto full_c, auto ext_c) {
             constexpr bool full = decltype(full_c)::value;
+            constexpr bool ext = decltype(ext_c)::value;  // the largest |MO| is wanted
             const int cnt = full ? G : N - d0;
             const T* st = acquire();
-            // boundary test W^2 inv_scale^2 - b^2 > 0 (MO^2 > b^2): its maximum over
-            // the batch, the first crossing searched only in a batch that has one
-            float cv[G], blk = 0.f, cmax = -INFINITY;
+            const uint32_t bits = mask_bits(d0, n);
+            const float J0 = Jf;
+            float Wu[G], blk = 0.f, amax = 0.f;
 #pragma unroll
             for (int u = 0; u < G; ++u) {
                 float y;
-                const float v = get(st, d0, u, cnt, full, y);
+                const float v = get(st, bits, u, cnt, full, y);
                 const bool take = v != 0.f;
                 const float r =
                     residual2<K>(y, sXm + (full ? d0 + u - n : min(d0 + u, N - 1) - n) * K, bres, lo0, lo1);
                 const float old = ring[slot * kThreads];
-                const float ro = Jf > (float)(np + 1) ? old : 0.f;
                 if (take) ring[slot * kThreads] = r;
                 const int nslot = slot + 1 == hp ? 0 : slot + 1;
                 slot = take ? nslot : slot;
-                const float Wn = (W + r) - ro;
+                const float Wn = (W + r) - old;
                 W = take ? Wn : W;
-                const float b2 = Jf > jlimf ? fmaf(lam2ln2, log2_fast(Jf), -blg) : P.lam2;
-                const float c = take ? fmaf(W * W, inv2, -b2) : -1.f;
-                cv[u] = c;
-                cmax = fmaxf(cmax, c);
+                Wu[u] = W;
+                amax = fmaxf(amax, fabsf(W));
                 blk += take ? W : 0.f;
-                wmax = take ? fmaxf(wmax, W) : wmax;
-                wmin = take ? fminf(wmin, W) : wmin;
+                if (ext) {
+                    wmax = take ? fmaxf(wmax, W) : wmax;
+                    wmin = take ? fminf(wmin, W) : wmin;
+                }
                 Jf += v;
             }
-            if (brk < 0 && cmax > 0.f) {
+            // boundary test W^2 inv_scale^2 - b^2 > 0 (MO^2 > b^2).  The boundary grows with the
+            // position: a batch whose largest |MO| stays within it at its first position holds
+            // no crossing (lowered by 1e-5, more than its rounding, so that none is missed),
+            // and the dates are tested only in the others, until the first crossing.  Testing
+            // every date cost a logarithm and six more operations a date.
+            if (brk < 0) {
+                auto bound = [&](float J) { return J > jlimf ? fmaf(lam2ln2, log2_fast(J), -blg) : P.lam2; };
+                if (fmaf(amax * amax, inv2, -(bound(J0) * 0.99999f)) > 0.f) {
+                    float J = J0;
 #pragma unroll
-                for (int u = 0; u < G; ++u)
-                    if (brk < 0 && cv[u] > 0.f) brk = d0 + u;
+                    for (int u = 0; u < G; ++u) {
+                        float y;
+                        if (get(st, bits, u, cnt, full, y) != 0.f) {
+                            if (brk < 0 && fmaf(Wu[u] * Wu[u], inv2, -bound(J)) > 0.f) brk = d0 + u;
+                            J += 1.f;
+                        }
+                    }
+                }
             }
             comp_add(sh, sl, blk);
             release();
         };
-        for (d0 = n; d0 + G <= N && !bad; d0 += G) passC(d0, std::true_type{});
-        if (d0 < N && !bad) passC(d0, std::false_type{});
+        if (kMask) mb.open(n, lane);
+        d0 = n;
+        if (P.maxmo) {
+            for (; d0 + G <= N && !bad; d0 += G) passC(d0, std::true_type{}, std::true_type{});
+            if (d0 < N && !bad) passC(d0, std::false_type{}, std::true_type{});
+        } else {
+            for (; d0 + G <= N && !bad; d0 += G) passC(d0, std::true_type{}, std::false_type{});
+            if (d0 < N && !bad) passC(d0, std::false_type{}, std::false_type{});
+        }
         if (bad) break;
         if (!active) continue;
 
@@ -573,7 +651,7 @@ bfm_status launch_stream(const bfm_design_s* d, int dtype, const void* Y, const 
     const int per_sm = 2.0 * kThreads * n_hist * (double)elt * sms <= kL2Budget ? 2 : 1;
     const int64_t ntiles = (m + kThreads - 1) / kThreads;
     const int grid = (int)(ntiles < (int64_t)per_sm * sms ? ntiles : (int64_t)per_sm * sms);
-    const size_t smem = stream_layout(d->N, n_hist, d->K, basis_stride(d->k), P.hmax).total;
+    const size_t smem = stream_layout(d->N, n_hist, d->K, basis_stride(d->k), P.hmax).bars + kBarBytes;
     if (d->k == 1) return launch_kh<1>(tm, P, dtype, grid, smem, stream);
     if (d->k == 2) return launch_kh<2>(tm, P, dtype, grid, smem, stream);
     return launch_kh<3>(tm, P, dtype, grid, smem, stream);
