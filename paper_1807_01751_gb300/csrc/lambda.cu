@@ -23,7 +23,8 @@
 // most; in FP64 by 6.6e-16 and 4.8e-15.  Fixed-point sums do not
 // depend on their order, so a warp takes one path, 32 steps at a time: every lane
 // draws one step, a prefix sum over the warp gives W, and the last h G of them
-// stay in a shared-memory ring for W(t - h): 4.3 ms.
+// stay in a shared-memory ring for W(t - h): 4.3 ms, and 3.9 with the quantile
+// taken on the device.
 #include <algorithm>
 #include <cmath>
 #include <mutex>
@@ -73,6 +74,47 @@ __device__ __forceinline__ int64_t warp_scan(int64_t v, int lane) {  // inclusiv
         v += lane >= o ? t : 0;
     }
     return v;
+}
+
+// The k-th smallest (from 0) of n values >= 0 into v[n]: their bits order as the values
+// do, and one block fixes eleven of them at a time from the top, counting the values
+// that share the bits fixed so far.  A host nth_element took 0.9 ms for 1e5 values.
+constexpr int kSelThreads = 1024, kSelBits = 11;
+__global__ void __launch_bounds__(kSelThreads) kth_smallest(double* v, int n, int k) {
+    __shared__ int hist[1 << kSelBits];
+    __shared__ int s_digit, s_below;
+    uint64_t prefix = 0;
+    for (int top = 64; top > 0; top -= kSelBits) {
+        const int shift = top > kSelBits ? top - kSelBits : 0, width = top - shift;
+        for (int i = threadIdx.x; i < (1 << kSelBits); i += kSelThreads) hist[i] = 0;
+        __syncthreads();
+        for (int i = threadIdx.x; i < n; i += kSelThreads) {
+            const uint64_t u = (uint64_t)__double_as_longlong(v[i]);
+            if (top == 64 || (u >> top) == (prefix >> top)) atomicAdd(&hist[(int)((u >> shift) & ((1u << width) - 1u))], 1);
+        }
+        __syncthreads();
+        if (threadIdx.x < 32) {  // 64 counts a lane
+            constexpr int kEach = (1 << kSelBits) / 32;
+            int sum = 0;
+            for (int i = 0; i < kEach; ++i) sum += hist[threadIdx.x * kEach + i];
+            int below = 0;  // values in the lanes before
+            for (int l = 0; l < 32; ++l) {
+                const int t = __shfl_sync(~0u, sum, l);
+                below += l < (int)threadIdx.x ? t : 0;
+            }
+            if (k >= below && k < below + sum) {
+                int d = threadIdx.x * kEach;
+                for (; k >= below + hist[d]; ++d) below += hist[d];
+                s_digit = d;
+                s_below = below;
+            }
+        }
+        __syncthreads();
+        prefix |= (uint64_t)s_digit << shift;
+        k -= s_below;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) v[n] = __longlong_as_double((long long)prefix);
 }
 
 // One path per warp.  kRing: W(t - h) from the ring; otherwise (h G too long for
@@ -192,7 +234,7 @@ extern "C" bfm_status bfm_lambda(double alpha, double h, double T, int G, int re
     }
     cudaStream_t st = (cudaStream_t)stream;
     double* d_stats = nullptr;
-    cudaError_t e = cudaMallocAsync(&d_stats, sizeof(double) * (size_t)reps, st);
+    cudaError_t e = cudaMallocAsync(&d_stats, sizeof(double) * ((size_t)reps + 1), st);
     if (e != cudaSuccess) return cuda_fail(e, "bfm_lambda: cudaMallocAsync");
     LambdaParams P{};
     P.G = G;
@@ -213,17 +255,20 @@ extern "C" bfm_status bfm_lambda(double alpha, double h, double T, int G, int re
     const bool ring = (size_t)slots * kWarps * 8 <= kMaxRingBytes;
     P.ring = ring ? (int)slots : 0;
     e = ring ? launch_paths<true>(P, (size_t)slots * kWarps * 8, st) : launch_paths<false>(P, 0, st);
-    std::vector<double> stats((size_t)reps);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(stats.data(), d_stats, sizeof(double) * (size_t)reps, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaFreeAsync(d_stats, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return cuda_fail(e, "bfm_lambda: simulation");
-    if (stats_host) std::copy(stats.begin(), stats.end(), stats_host);
     // (1 - alpha) empirical quantile: the ceil((1 - alpha) reps)-th smallest
     long q = (long)std::ceil((1.0 - alpha) * (double)reps) - 1;
     q = q < 0 ? 0 : (q >= reps ? reps - 1 : q);
-    std::nth_element(stats.begin(), stats.begin() + q, stats.end());
-    *lambda_out = stats[(size_t)q];
+    if (e == cudaSuccess) {
+        kth_smallest<<<1, kSelThreads, 0, st>>>(d_stats, reps, (int)q);
+        e = cudaGetLastError();
+    }
+    double lambda = 0.0;
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&lambda, d_stats + reps, sizeof lambda, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess && stats_host)
+        e = cudaMemcpyAsync(stats_host, d_stats, sizeof(double) * (size_t)reps, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaFreeAsync(d_stats, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return cuda_fail(e, "bfm_lambda: simulation");
+    *lambda_out = lambda;
     return BFM_OK;
 }
