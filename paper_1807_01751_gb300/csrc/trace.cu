@@ -26,7 +26,8 @@
 // solving in every lane alike took about 2400 per warp and pixel: 709 us for 4096
 // pixels of 414 dates.  Now the regressors are read from the design's table, the
 // sums are folded (each exchange halves the values a lane carries) and the
-// factorisation is spread over the lanes: about 400, 178 us.
+// factorisation is spread over the lanes: about 400, 178 us; with runs of the prefix sums per lane and no division per
+// date, 160 us.
 #include <cmath>
 
 #include "bfm_internal.cuh"
@@ -258,29 +259,36 @@ __global__ void __launch_bounds__(32 * kMaxWarps) trace_kernel(const TraceParams
     if (!mo_row) return;
     __syncwarp();
 
-    // 4. prefix sums of the residuals in place, then the windows of h_p terms
-    double carry = 0.0;
-    for (int j0 = 0; j0 < nv; j0 += 32) {
-        const int j = j0 + lane;
-        double v = j < nv ? val[j] : 0.0;
+    // 4. prefix sums of the residuals in place (a run of consecutive ones per lane, then the
+    // lanes' totals), then the windows of h_p terms
+    {
+        const int c = (nv + 31) / 32, j0 = lane * c, j1 = min(j0 + c, nv);
+        double run = 0.0;
+        for (int j = j0; j < j1; ++j) {
+            run += val[j];
+            val[j] = run;
+        }
+        double before = run;
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
-            const double u = __shfl_up_sync(~0u, v, off);
-            if (lane >= off) v += u;
+            const double u = __shfl_up_sync(~0u, before, off);
+            if (lane >= off) before += u;
         }
-        v += carry;
-        if (j < nv) val[j] = v;
-        carry = __shfl_sync(~0u, v, 31);
+        before = __shfl_up_sync(~0u, before, 1);
+        if (lane > 0)
+            for (int j = j0; j < j1; ++j) val[j] += before;
     }
     __syncwarp();
     int hp = (int)floor(P.h_frac * (double)np);
     hp = hp < 1 ? 1 : (hp > np ? np : hp);
-    const double scale = sqrt(ss / (double)(np - K)) * sqrt((double)np);
+    const double inv_scale = 1.0 / (sqrt(ss / (double)(np - K)) * sqrt((double)np));
     const bool degenerate = st == BFM_PX_DEGENERATE;
     for (int t = lane; t < N; t += 32) {
-        const int q = pos[t];  // 0-based position: the window holds positions q-hp+1..q
         float out = qnan;
-        if (q >= np) out = degenerate ? 0.0f : (float)((val[q] - val[q - hp]) / scale);
+        if (t >= P.n_hist) {
+            const int q = pos[t];  // 0-based position: the window holds positions q-hp+1..q
+            if (q >= np) out = degenerate ? 0.0f : (float)((val[q] - val[q - hp]) * inv_scale);
+        }
         mo_row[t] = out;
     }
 }
