@@ -217,15 +217,16 @@ bfm_status bfm_monitor_ext(bfm_design_t d, const void *Y, int dtype, const uint3
  * lambda*sqrt(log+(t)) (Eq. 4), found by simulation of the limiting process
  * as the paper prescribes (Section 2.3; Section 4.3 prints 2.39 for
  * alpha = 0.05, h = 0.5, N/n = 2).  `reps` Brownian paths on a grid of G
- * steps per unit time up to T = N/n (T * G steps, rounded), one per GPU
- * thread, each from its own SplitMix64 stream (path r: state
+ * steps per unit time up to T = N/n (T * G steps, rounded), each from its
+ * own SplitMix64 stream (path r: state
  * seed * 0xA0761D6478BD642F + r * 0xE7037ED1A0B428DB + 1, one draw
  * discarded) with Box-Muller normals; the statistic of a path is
  * sup over t = i/G in [1, T] of |W(t) - W(t-h) - h W(1)| / sqrt(log+ t),
  * with h rounded to whole steps.  *lambda_out receives the
  * ceil((1 - alpha) * reps)-th smallest statistic; stats_host (nullable,
  * host, reps doubles) receives all of them.  Runs on `stream` and returns
- * when done (synchronising it).  FP64 arithmetic.
+ * when done (synchronising it).  The paths are 64-bit fixed-point words whose
+ * step is finer than the rounding of a double; the results are doubles.
  * Errors: BFM_EINVAL (0 < alpha < 1, 0 < h <= 1, T > 1, G >= 1, reps >= 1
  * and round(h * G) >= 1 are required), BFM_ECUDA.
  */

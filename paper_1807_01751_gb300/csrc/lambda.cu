@@ -19,12 +19,13 @@
 // took 52.6 ms, nearly all of it FP64 issue.  Here the normals come from
 // lambda_fixed.cuh (integer arithmetic) and W is a 64-bit fixed-point word, whose
 // step 2^-frac is finer than the rounding of an FP64 W: against 113-bit arithmetic,
-// over 150 such paths, the statistic is off by 1.1e-16 on average and 4.2e-16 at
+// over 150 such paths, the statistic is off by 7.3e-17 on average and 2.8e-16 at
 // most; in FP64 by 6.6e-16 and 4.8e-15.  Fixed-point sums do not
 // depend on their order, so a warp takes one path, 32 steps at a time: every lane
 // draws one step, a prefix sum over the warp gives W, and the last h G of them
-// stay in a shared-memory ring for W(t - h): 4.3 ms, and 3.9 with the quantile
-// taken on the device.
+// stay in a shared-memory ring for W(t - h): 3.6 ms, bound by the integer
+// pipe (4.3 before the quantile was taken on the device and the logarithm's sum kept in
+// one word).
 #include <algorithm>
 #include <cmath>
 #include <mutex>
@@ -46,7 +47,7 @@ struct LambdaParams {
     int ie;                // last step with log+ (i / G) = 1
     int ring;              // ring slots per warp (a multiple of 32, >= ih + 32), 0: no ring
     int frac;              // fraction bits of W
-    uint64_t seed, sd, h;  // sd, h: 1/sqrt(G) and h times 2^64 (h = 1 as 0)
+    uint64_t seed, sd, h;  // sd: sqrt(2 / G) 2^63; h times 2^64 (h = 1 as 0)
     double* stats;
 };
 
@@ -60,7 +61,7 @@ __device__ __forceinline__ uint64_t splitmix_mix(uint64_t z) {
 __device__ __forceinline__ int64_t increment(uint64_t s, const LambdaParams& P, const uint64_t* ln, const uint32_t* rec) {
     const uint64_t n = (splitmix_mix(s + kGolden) >> 11) + 1, f = splitmix_mix(s + 2 * kGolden) >> 11;
     bool neg;
-    const uint64_t z = fixedpt::normal_q58(n, f, ln, rec, neg);     // |z| <= 8.6
+    const uint64_t z = fixedpt::normal_q59(n, f, ln, rec, neg);     // 2^59 |z| / sqrt(2), |z| <= 8.6
     const uint64_t q = fixedpt::mulhi(z << 2, P.sd);                // 2^60 |z| / sqrt(G)
     const int sh = 60 - P.frac;
     const int64_t d = (int64_t)((q + (1ull << (sh - 1))) >> sh);
@@ -248,7 +249,7 @@ extern "C" bfm_status bfm_lambda(double alpha, double h, double T, int G, int re
     // three times that: the integer part holds 40 sqrt(T)
     P.frac = 62 - (int)std::ceil(std::log2(40.0 * std::sqrt(T)));
     P.seed = seed;
-    P.sd = G == 1 ? ~0ull : (uint64_t)std::ldexp(1.0 / std::sqrt((double)G), 64);
+    P.sd = (uint64_t)std::ldexp(std::sqrt(2.0 / (double)G), 63);
     P.h = h < 1.0 ? (uint64_t)std::ldexp(h, 64) : 0ull;
     P.stats = d_stats;
     const int64_t slots = ((int64_t)ih + 63) / 32 * 32;

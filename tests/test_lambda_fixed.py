@@ -1,11 +1,10 @@
 """The fixed-point Box-Muller normal of the critical-value simulation
 (csrc/lambda_fixed.cuh) on the host, against 50-digit decimal arithmetic.
 
-Bound: -2 ln u is off by at most 2^-57 (53 roundings of ln 2 at 2^-65, a table
-entry and a series at a few 2^-64, doubled), so its root by at most 2^-57 / 2 /
-2^-5.5 where u < 1 - 2^-12; nearer to 1 the logarithm is FP64, 2^-53 relative.
-The cosine and the product add a few 2^-58: 2^-52 in all, the rounding of an
-FP64 value of magnitude 2.
+The function returns |z| / sqrt(2).  Bound: -ln u is truncated to 2^-58 in three
+terms, so its root is off by at most 2^-56.4 / 2 / 2^-6 where u < 1 - 2^-12;
+nearer to 1 the logarithm is FP64, 2^-53 relative.  The cosine and the product
+add a few 2^-59: 2^-51 in all, the rounding of an FP64 value of magnitude 4.
 """
 import ctypes
 import os
@@ -21,7 +20,7 @@ SRC = """
 #define __device__
 #define __forceinline__ inline
 #include "lambda_fixed.cuh"
-extern "C" long long normal_q58(unsigned long long n, unsigned long long f) {
+extern "C" long long normal_q59(unsigned long long n, unsigned long long f) {
     using namespace bfm::fixedpt;
     static uint64_t ln[256];
     static uint32_t rec[256];
@@ -31,7 +30,7 @@ extern "C" long long normal_q58(unsigned long long n, unsigned long long f) {
             rec[i] = log_recip(i);
         }
     bool neg;
-    const uint64_t z = normal_q58(n, f, ln, rec, neg);
+    const uint64_t z = normal_q59(n, f, ln, rec, neg);
     return neg ? -(long long)z : (long long)z;
 }
 """
@@ -45,7 +44,7 @@ def normal(tmp_path_factory):
     so = str(d / "n.so")
     subprocess.check_call(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I",
                            os.path.join(ROOT, "paper_1807_01751_gb300", "csrc"), str(d / "n.cpp"), "-o", so])
-    f = ctypes.CDLL(so).normal_q58
+    f = ctypes.CDLL(so).normal_q59
     f.argtypes, f.restype = [ctypes.c_uint64, ctypes.c_uint64], ctypes.c_int64
     return f
 
@@ -73,8 +72,8 @@ def test_normals(normal):
     for i, n in enumerate(ns):
         f = fs[i % len(fs)] if i % 3 == 0 else r.randrange(top)
         x = Decimal(f) / top
-        ref = (-2 * (Decimal(n) / top).ln()).sqrt() * cosine(2 * PI * (x if x <= Decimal(0.5) else 1 - x))
-        err = abs(Decimal(normal(n, f)) / 2 ** 58 - ref)
-        assert err <= Decimal(2) ** -52, (n, f, float(err))
+        ref = (-(Decimal(n) / top).ln()).sqrt() * cosine(2 * PI * (x if x <= Decimal(0.5) else 1 - x))
+        err = abs(Decimal(normal(n, f)) / 2 ** 59 - ref)
+        assert err <= Decimal(2) ** -51, (n, f, float(err))
         total += err
     assert total / len(ns) < Decimal(2) ** -55
