@@ -90,8 +90,9 @@ constexpr int kStages = 3;                // stages in flight per group
 // stages and barriers: the four pixel warps of a scheduler then belong to two
 // pipelines, and one computes while the other waits for a stage, an MMA or a solve.
 // With all four M-tiles in one group the kernel issued on 58 % of its cycles, with two
-// groups 68 %: 7.50 -> 6.68 ms (float) and 7.63 -> 6.95 ms (int16) on 8.4 Mi pixels of 414
-// dates, 193 -> 170 us on 250k pixels of 256.  One M-tile per group (24 warps, 80
+// groups 68 %: 7.50 -> 6.70 ms (float) and 7.63 -> 6.91 ms (int16) on 8.4 Mi pixels of 414
+// dates, 193 -> 167 us on 250k pixels of 256; with whole chunks and groups in loops of
+// their own, without bounds checks, 6.48 ms, 6.49 ms and 154 us.  One M-tile per group (24 warps, 80
 // registers) was slower at every size but the smallest.
 constexpr int kGrp = 2;                       // M-tiles per group
 constexpr int kGroups = kMT / kGrp;
@@ -424,14 +425,14 @@ __device__ __forceinline__ void mon_step(bool ok, float r, float* ring_t, Mon& m
     }
 }
 
-// Monitoring dates [d8, d8 + 8), all >= n (kFull: all < N).
-template <bool kFull, bool kExt, typename T, bool kMask>
-__device__ __forceinline__ void mon8(const Obs<T, kMask>& ob, const T (&raw)[8], int d8, int N, const float* yh,
-                                     float* ring_t, Mon& mo, float (&Wu)[8]) {
+// Eight monitoring dates, all in [n, N).
+template <bool kExt, typename T, bool kMask>
+__device__ __forceinline__ void mon8(const Obs<T, kMask>& ob, const T (&raw)[8], const float* yh, float* ring_t,
+                                     Mon& mo, float (&Wu)[8]) {
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
         bool ok;
-        const float y = ob.value(raw[u], u, kFull || d8 + u < N, ok);
+        const float y = ob.value(raw[u], u, true, ok);
         mon_step<kExt>(ok, fmaf(-yh[u], mo.inv_sb, y), ring_t, mo);
         Wu[u] = mo.W;
     }
@@ -888,7 +889,10 @@ __global__ void __launch_bounds__(kThreads, 1)
             // ---- pass A: A operands of the masked basis sums and X'My
             float ymax = 0.f;
             if (kMask) mb.open(0, lane);
-            for (int c = 0; c < nck && !bad; ++c) {
+            // whole chunks carry no bounds checks; the last dates of a history that ends
+            // within a chunk go through the same code with them
+            auto chunk_a = [&](int c, auto full_c) {
+                constexpr bool full = decltype(full_c)::value;
                 const uint32_t b = cc & 1u;
                 if (kMask && (c & 1) == 0) mb.next(16 * c, lane);
                 uint32_t yv[16], mk[8];
@@ -896,17 +900,14 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const int d8 = 16 * c + 8 * h;
-                    if (d8 < n) {  // warp-uniform: the dates exist
+                    if (full || d8 < n) {  // warp-uniform: the dates exist
                         if (h == 0 || G == 8) stg = acquire();
                         const T* st = stg + (G == 16 ? h * 8 * kBoxPx : 0);
                         if (kMask) ob.bits = mb.cur >> (d8 & 31);
                         T raw[8];
                         load8(st, raw);
-                        if (d8 + 8 <= n)
-                            pass_a8<true>(ob, raw, d8, n, yv + 8 * h, mk + 4 * h, ymax);
-                        else
-                            pass_a8<false>(ob, raw, d8, n, yv + 8 * h, mk + 4 * h, ymax);
-                        if (G == 8 || h == 1 || d8 + 8 >= n) release();
+                        pass_a8<full>(ob, raw, d8, n, yv + 8 * h, mk + 4 * h, ymax);
+                        if (G == 8 || h == 1 || (!full && d8 + 8 >= n)) release();
                     } else {
 #pragma unroll
                         for (int u = 0; u < 8; ++u) yv[8 * h + u] = 0u;
@@ -914,8 +915,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                         for (int j = 0; j < 4; ++j) mk[4 * h + j] = 0u;
                     }
                 }
-                if (bad) break;
-                if (cc >= 2 && !wait_w(aempty + b, ((cc >> 1) - 1) & 1u)) break;
+                if (bad || (cc >= 2 && !wait_w(aempty + b, ((cc >> 1) - 1) & 1u))) return;
                 ptx::tc_fence_after();
                 const uint32_t a = tl + tcol + kColA + 24u * b;
                 ptx::tmem_st8(a, mk);
@@ -923,7 +923,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                 ptx::tmem_wait_st();
                 arrive(afull + b);
                 ++cc;
-            }
+            };
+            const int nwhole = n / 16;
+            for (int c = 0; c < nwhole && !bad; ++c) chunk_a(c, std::true_type{});
+            if (nwhole < nck && !bad) chunk_a(nwhole, std::false_type{});
             if (bad) break;
             if (!wait_w(accd, 0u)) break;
             ptx::tc_fence_after();
@@ -998,9 +1001,10 @@ __global__ void __launch_bounds__(kThreads, 1)
             float ss0 = 0.f;
             int rem = wq, wdate = n;
             if (kMask) mb.open(0, lane);
-            for (int c = 0; c < nck && !bad; ++c) {
+            auto chunk_b = [&](int c, auto full_c) {
+                constexpr bool full = decltype(full_c)::value;
                 if (kMask && (c & 1) == 0) mb.next(16 * c, lane);
-                if (!wait_w(yfull + (pc & 1u), (pc >> 1) & 1u)) break;
+                if (!wait_w(yfull + (pc & 1u), (pc >> 1) & 1u)) return;
                 ptx::tc_fence_after();
                 uint32_t yq[2][8];
                 ptx::tmem_ld8_issue(tl + tcol + kColY0 + 16u * (pc & 1u), yq[0]);
@@ -1011,7 +1015,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const int d8 = 16 * c + 8 * h;
-                    if (d8 < n) {
+                    if (full || d8 < n) {
                         if (h == 0 || G == 8) stg = acquire();
                         const T* st = stg + (G == 16 ? h * 8 * kBoxPx : 0);
                         if (kMask) ob.bits = mb.cur >> (d8 & 31);
@@ -1026,24 +1030,12 @@ __global__ void __launch_bounds__(kThreads, 1)
                         float yh[8];
 #pragma unroll
                         for (int u = 0; u < 8; ++u) yh[u] = __uint_as_float(yq[h][u]);
-                        const bool scan = __any_sync(~0u, rem < 8);  // a pixel may reach its window start
-                        const bool fullb = d8 + 8 <= n;
-                        if (scan) {
-                            if (fullb)
-                                pass_b8<true, true>(ob, raw, d8, n, yh, inv_fit, s_r, ss0, hw + 4 * h,
-                                                    lw + 4 * h, rem, wdate);
-                            else
-                                pass_b8<false, true>(ob, raw, d8, n, yh, inv_fit, s_r, ss0, hw + 4 * h,
-                                                     lw + 4 * h, rem, wdate);
-                        } else {
-                            if (fullb)
-                                pass_b8<true, false>(ob, raw, d8, n, yh, inv_fit, s_r, ss0, hw + 4 * h,
-                                                     lw + 4 * h, rem, wdate);
-                            else
-                                pass_b8<false, false>(ob, raw, d8, n, yh, inv_fit, s_r, ss0, hw + 4 * h,
-                                                      lw + 4 * h, rem, wdate);
-                        }
-                        if (G == 8 || h == 1 || d8 + 8 >= n) release();
+                        // a pixel may reach its window's start among these dates (after it, rem < 0)
+                        if (!full || __any_sync(~0u, (unsigned)rem < 8u))
+                            pass_b8<full, true>(ob, raw, d8, n, yh, inv_fit, s_r, ss0, hw + 4 * h, lw + 4 * h, rem, wdate);
+                        else
+                            pass_b8<full, false>(ob, raw, d8, n, yh, inv_fit, s_r, ss0, hw + 4 * h, lw + 4 * h, rem, wdate);
+                        if (G == 8 || h == 1 || (!full && d8 + 8 >= n)) release();
                     } else {
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
@@ -1052,8 +1044,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                         }
                     }
                 }
-                if (bad) break;
-                if (cc >= 2 && !wait_w(aempty + b, ((cc >> 1) - 1) & 1u)) break;
+                if (bad || (cc >= 2 && !wait_w(aempty + b, ((cc >> 1) - 1) & 1u))) return;
                 ptx::tc_fence_after();
                 const uint32_t a = tl + tcol + kColR + 16u * b;
                 ptx::tmem_st8(a, hw);
@@ -1061,7 +1052,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                 ptx::tmem_wait_st();
                 arrive(afull + b);
                 ++cc;
-            }
+            };
+            for (int c = 0; c < nwhole && !bad; ++c) chunk_b(c, std::true_type{});
+            if (nwhole < nck && !bad) chunk_b(nwhole, std::false_type{});
             if (bad) break;
             if (!wait_w(accd, 1u)) break;
             ptx::tc_fence_after();
@@ -1164,68 +1157,93 @@ __global__ void __launch_bounds__(kThreads, 1)
             float sh = 0.f, sl = 0.f;
             const T* stg = nullptr;
             if (kMask) mb.open(ds, lane);
-            for (int d8 = ds; d8 < N && !bad; d8 += 8) {
+            // the values and fitted values of the dates [d8, d8 + 8); a stage or a piece of
+            // fitted values is handed back behind its last group (end8, and here)
+            auto begin8 = [&](int d8, T (&raw)[8], float (&yh)[8]) -> bool {
                 const int off = d8 - ds;
                 if (kMask) {
                     if ((off & 31) == 0) mb.next(d8, lane);
                     ob.bits = mb.cur >> (off & 31);
                 }
-                if ((off & 31) == 0 && !wait_w(yfull + (pc & 1u), (pc >> 1) & 1u)) break;
+                if ((off & 31) == 0 && !wait_w(yfull + (pc & 1u), (pc >> 1) & 1u)) return false;
                 ptx::tc_fence_after();
                 uint32_t yq[8];
                 ptx::tmem_ld8_issue(tl + tcol + kColY + 32u * (pc & 1u) + (uint32_t)(off & 31), yq);
-                if (off % G == 0) {
-                    stg = acquire();
-                }
-                const T* st8 = stg + (off % G) * kBoxPx;  // dates of the stage are rows of kBoxPx elements
-                T raw[8];
-                load8(st8, raw);
+                if (off % G == 0) stg = acquire();
+                load8(stg + (off % G) * kBoxPx, raw);  // dates of the stage are rows of kBoxPx elements
                 ptx::tmem_wait_ld8(yq);
-                float yh[8];
 #pragma unroll
                 for (int u = 0; u < 8; ++u) yh[u] = __uint_as_float(yq[u]);
                 if ((off & 31) == 24 || d8 + 8 >= N) {
                     arrive(yempty + (pc & 1u));
                     ++pc;
                 }
-                if (d8 + 8 <= n) {
-                    mon_hist8(ob, raw, d8, yh, ring_t, mo);
-                } else {
-                    const int J0 = np + 1 + mo.cnt;
-                    float Wu[8];
-                    mo.blk = 0.f;
-                    mo.amax = 0.f;
-                    if (d8 >= n && d8 + 8 <= N) {
-                        if (maxmo)
-                            mon8<true, true>(ob, raw, d8, N, yh, ring_t, mo, Wu);
-                        else
-                            mon8<true, false>(ob, raw, d8, N, yh, ring_t, mo, Wu);
-                    } else {
-                        mon_mixed8(ob, raw, d8, n, N, yh, ring_t, mo, Wu, maxmo != nullptr);
-                    }
-                    comp_add(sh, sl, mo.blk);
-                    // the boundary grows with the position: a stretch whose largest |MO| stays
-                    // within the boundary at its first position holds no crossing (lowered by
-                    // 1e-6 relative, so that rounding of the boundary never hides a crossing)
-                    if (brk < 0) {
-                        const float Jf0 = (float)J0;
-                        const float b2f = (Jf0 > jlimf ? fmaf(lam2ln2, log2_fast(Jf0), -blg) : lam2) * 0.999999f;
-                        if (fmaf(mo.amax * mo.amax, inv2, -b2f) > 0.f) {
-                            float Jc = Jf0;
+                return true;
+            };
+            auto end8 = [&](int d8) {
+                if (((d8 - ds) % G) + 8 == G || d8 + 8 >= N) release();
+            };
+            // the boundary grows with the position: a stretch whose largest |MO| stays
+            // within the boundary at its first position J0 holds no crossing (lowered by
+            // 1e-6 relative, so that rounding of the boundary never hides a crossing)
+            auto test8 = [&](int d8, int J0, const T (&raw)[8], const float (&Wu)[8]) {
+                comp_add(sh, sl, mo.blk);
+                if (brk < 0) {
+                    const float Jf0 = (float)J0;
+                    const float b2f = (Jf0 > jlimf ? fmaf(lam2ln2, log2_fast(Jf0), -blg) : lam2) * 0.999999f;
+                    if (fmaf(mo.amax * mo.amax, inv2, -b2f) > 0.f) {
+                        float Jc = Jf0;
 #pragma unroll
-                            for (int u = 0; u < 8; ++u) {
-                                const int d = d8 + u;
-                                if (d >= n && ob.valid(raw[u], u, d < N)) {
-                                    const float b2 = Jc > jlimf ? fmaf(lam2ln2, log2_fast(Jc), -blg) : lam2;
-                                    if (brk < 0 && fmaf(Wu[u] * Wu[u], inv2, -b2) > 0.f) brk = d;
-                                    Jc += 1.f;
-                                }
+                        for (int u = 0; u < 8; ++u) {
+                            const int d = d8 + u;
+                            if (d >= n && ob.valid(raw[u], u, d < N)) {
+                                const float b2 = Jc > jlimf ? fmaf(lam2ln2, log2_fast(Jc), -blg) : lam2;
+                                if (brk < 0 && fmaf(Wu[u] * Wu[u], inv2, -b2) > 0.f) brk = d;
+                                Jc += 1.f;
                             }
                         }
                     }
                 }
-                if ((off % G) + 8 == G || d8 + 8 >= N) release();
+            };
+            // eight dates that hold n or N
+            auto mixed = [&](int d8) -> bool {
+                T raw[8];
+                float yh[8], Wu[8];
+                if (!begin8(d8, raw, yh)) return false;
+                const int J0 = np + 1 + mo.cnt;
+                mo.blk = 0.f;
+                mo.amax = 0.f;
+                mon_mixed8(ob, raw, d8, n, N, yh, ring_t, mo, Wu, maxmo != nullptr);
+                test8(d8, J0, raw, Wu);
+                end8(d8);
+                return true;
+            };
+            auto monitor8 = [&](int d8, auto ext_c) -> bool {
+                T raw[8];
+                float yh[8], Wu[8];
+                if (!begin8(d8, raw, yh)) return false;
+                const int J0 = np + 1 + mo.cnt;
+                mo.blk = 0.f;
+                mo.amax = 0.f;
+                mon8<decltype(ext_c)::value>(ob, raw, yh, ring_t, mo, Wu);
+                test8(d8, J0, raw, Wu);
+                end8(d8);
+                return true;
+            };
+            int d8 = ds;
+            for (; d8 + 8 <= n && !bad; d8 += 8) {
+                T raw[8];
+                float yh[8];
+                if (!begin8(d8, raw, yh)) break;
+                mon_hist8(ob, raw, d8, yh, ring_t, mo);
+                end8(d8);
             }
+            if (d8 < n && !bad && mixed(d8)) d8 += 8;
+            if (maxmo)
+                for (; d8 + 8 <= N && !bad && monitor8(d8, std::true_type{}); d8 += 8) {}
+            else
+                for (; d8 + 8 <= N && !bad && monitor8(d8, std::false_type{}); d8 += 8) {}
+            if (d8 < N && !bad) mixed(d8);
             if (bad) break;
             if (!active) continue;
 
