@@ -19,13 +19,13 @@
 // took 52.6 ms, nearly all of it FP64 issue.  Here the normals come from
 // lambda_fixed.cuh (integer arithmetic) and W is a 64-bit fixed-point word, whose
 // step 2^-frac is finer than the rounding of an FP64 W: against 113-bit arithmetic,
-// over 150 such paths, the statistic is off by 7.3e-17 on average and 2.8e-16 at
+// over 150 such paths, the statistic is off by 7.2e-17 on average and 2.2e-16 at
 // most; in FP64 by 6.6e-16 and 4.8e-15.  Fixed-point sums do not
-// depend on their order, so a warp takes one path, 32 steps at a time: every lane
-// draws one step, a prefix sum over the warp gives W, and the last h G of them
-// stay in a shared-memory ring for W(t - h): 3.6 ms, bound by the integer
-// pipe (4.3 before the quantile was taken on the device and the logarithm's sum kept in
-// one word).
+// depend on their order, so a warp takes one path, 64 steps at a time: every lane
+// draws two, a prefix sum over the warp gives W, and the last h G of them
+// stay in a shared-memory ring for W(t - h): 3.5 ms, bound by the integer
+// pipe (4.3 before the quantile was taken on the device, the logarithm's sum kept in one
+// word and the additions of the 64-bit products folded into the multiplies).
 #include <algorithm>
 #include <cmath>
 #include <mutex>
@@ -39,13 +39,15 @@ namespace {
 
 constexpr uint64_t kGolden = 0x9E3779B97F4A7C15ull;  // SplitMix64 increment
 constexpr int kWarps = 4;                             // paths at a time per block
+constexpr int kPer = 2;                               // consecutive steps of a lane
+constexpr int kSteps = 32 * kPer;                     // steps of a warp at a time
 constexpr double kE = 2.718281828459045235360287;
 constexpr size_t kMaxRingBytes = 200 * 1024;          // rings of a block
 
 struct LambdaParams {
     int G, nsteps, ih, reps;
     int ie;                // last step with log+ (i / G) = 1
-    int ring;              // ring slots per warp (a multiple of 32, >= ih + 32), 0: no ring
+    int ring;              // ring slots per warp (a multiple of kSteps, >= ih + kSteps), 0: no ring
     int frac;              // fraction bits of W
     uint64_t seed, sd, h;  // sd: sqrt(2 / G) 2^63; h times 2^64 (h = 1 as 0)
     double* stats;
@@ -62,8 +64,8 @@ __device__ __forceinline__ int64_t increment(uint64_t s, const LambdaParams& P, 
     const uint64_t n = (splitmix_mix(s + kGolden) >> 11) + 1, f = splitmix_mix(s + 2 * kGolden) >> 11;
     bool neg;
     const uint64_t z = fixedpt::normal_q59(n, f, ln, rec, neg);     // 2^59 |z| / sqrt(2), |z| <= 8.6
-    const uint64_t q = fixedpt::mulhi(z << 2, P.sd);                // 2^60 |z| / sqrt(G)
-    const int sh = 60 - P.frac;
+    const uint64_t q = fixedpt::mulhi(z, P.sd);                     // 2^58 |z| / sqrt(G); sd < 1.5 2^63, z < 2^62
+    const int sh = 58 - P.frac;                                     // >= 2
     const int64_t d = (int64_t)((q + (1ull << (sh - 1))) >> sh);
     return neg ? -d : d;
 }
@@ -125,7 +127,7 @@ __global__ void __launch_bounds__(32 * kWarps)
     lambda_paths(const __grid_constant__ fixedpt::LogTable tab, const LambdaParams P) {
     __shared__ uint64_t s_ln[256];
     __shared__ uint32_t s_rec[256];
-    extern __shared__ int64_t s_ring[];
+    extern __shared__ __align__(16) int64_t s_ring[];
     for (int i = threadIdx.x; i < 256; i += 32 * kWarps) {
         s_ln[i] = tab.ln[i];
         s_rec[i] = fixedpt::log_recip((uint32_t)i);
@@ -137,8 +139,8 @@ __global__ void __launch_bounds__(32 * kWarps)
     for (int64_t r = (int64_t)blockIdx.x * kWarps + warp; r < P.reps; r += (int64_t)gridDim.x * kWarps) {
         // stream of path r (one discarded draw after seeding); step i uses draws 2i - 1 and 2i
         const uint64_t s0 = P.seed * 0xA0761D6478BD642Full + (uint64_t)r * 0xE7037ED1A0B428DBull + 1ull + kGolden;
-        uint64_t st = s0 + 2 * kGolden * (uint64_t)lane;
-        int64_t base = 0, hw1 = 0;  // W before the block of 32 steps, h W(1)
+        uint64_t st = s0 + 2 * kPer * kGolden * (uint64_t)lane;
+        int64_t base = 0, hw1 = 0;  // W before the block of steps, h W(1)
         int64_t lbase = 0;          // !kRing: W(t - h) before the block
         uint64_t best = 0;
         int pos = 0;                // ring slot of the block's first step
@@ -146,41 +148,57 @@ __global__ void __launch_bounds__(32 * kWarps)
             __syncwarp();  // the previous path's reads
             if (lane == 0) ring[P.ring - 1] = 0;  // W(0), the slot before step 1
         }
-        for (int i0 = 1; i0 <= P.nsteps; i0 += 32) {
-            const int i = i0 + lane;
-            const int64_t W = base + warp_scan(increment(st, P, s_ln, s_rec), lane);
-            st += 64 * kGolden;
-            base = __shfl_sync(~0u, W, 31);
-            int64_t lag = 0;
+        for (int i0 = 1; i0 <= P.nsteps; i0 += kSteps) {
+            const int i = i0 + kPer * lane;  // this lane's steps i, i + 1
+            int64_t W[kPer];
+            {
+                const int64_t d0 = increment(st, P, s_ln, s_rec), d1 = increment(st + 2 * kGolden, P, s_ln, s_rec);
+                W[1] = base + warp_scan(d0 + d1, lane);
+                W[0] = W[1] - d1;
+            }
+            st += 2 * kSteps * kGolden;
+            base = __shfl_sync(~0u, W[1], 31);
+            int64_t lag[kPer] = {0, 0};
             if (kRing) {
-                ring[pos + lane] = W;
+                *reinterpret_cast<longlong2*>(ring + pos + kPer * lane) = make_longlong2(W[0], W[1]);
                 __syncwarp();
-                int s = pos + lane - P.ih;
-                s += s < 0 ? P.ring : 0;
-                lag = ring[s];  // steps before the ring's first lap are not used (i < G)
-                pos += 32;
+#pragma unroll
+                for (int u = 0; u < kPer; ++u) {
+                    int s = pos + kPer * lane + u - P.ih;
+                    s += s < 0 ? P.ring : 0;
+                    lag[u] = ring[s];  // steps before the ring's first lap are not used (i < G)
+                }
+                pos += kSteps;
                 pos = pos == P.ring ? 0 : pos;
                 __syncwarp();
-            } else if (i0 + 31 > P.ih) {
-                const int j = i - P.ih;  // the lagged step
-                const int64_t inc = j >= 1 ? increment(s0 + 2 * kGolden * (uint64_t)(j - 1), P, s_ln, s_rec) : 0;
-                lag = lbase + warp_scan(inc, lane);
-                lbase = __shfl_sync(~0u, lag, 31);
+            } else if (i0 + kSteps - 1 > P.ih) {
+                int64_t d[kPer];  // the lagged steps
+#pragma unroll
+                for (int u = 0; u < kPer; ++u) {
+                    const int j = i + u - P.ih;
+                    d[u] = j >= 1 ? increment(s0 + 2 * kGolden * (uint64_t)(j - 1), P, s_ln, s_rec) : 0;
+                }
+                lag[1] = lbase + warp_scan(d[0] + d[1], lane);
+                lag[0] = lag[1] - d[1];
+                lbase = __shfl_sync(~0u, lag[1], 31);
             }
-            if (i0 + 31 >= P.G) {
+            if (i0 + kSteps - 1 >= P.G) {
                 if (i0 <= P.G) {  // W(1) is in this block
-                    const int64_t w1 = __shfl_sync(~0u, W, P.G - i0);
-                    const uint64_t a = (uint64_t)(w1 < 0 ? -w1 : w1), ha = P.h ? fixedpt::mulhi(a, P.h) : a;
+                    const int at = P.G - i0;
+                    const int64_t w1 = __shfl_sync(~0u, (at & 1) ? W[1] : W[0], at >> 1);
+                    const uint64_t a = (uint64_t)(w1 < 0 ? -w1 : w1), ha = P.h ? __umul64hi(a, P.h) : a;
                     hw1 = w1 < 0 ? -(int64_t)ha : (int64_t)ha;
                 }
-                if (i >= P.G && i <= P.nsteps) {
-                    const int64_t z = W - lag - hw1;
-                    uint64_t v = (uint64_t)(z < 0 ? -z : z);
-                    if (v > best) {  // the boundary's factor, at least 1, only lowers it
-                        if (i > P.ie) v = (uint64_t)((double)v / sqrt(log((double)i / (double)P.G)));
-                        best = v > best ? v : best;
+#pragma unroll
+                for (int u = 0; u < kPer; ++u)
+                    if (i + u >= P.G && i + u <= P.nsteps) {
+                        const int64_t z = W[u] - lag[u] - hw1;
+                        uint64_t v = (uint64_t)(z < 0 ? -z : z);
+                        if (v > best) {  // the boundary's factor, at least 1, only lowers it
+                            if (i + u > P.ie) v = (uint64_t)((double)v / sqrt(log((double)(i + u) / (double)P.G)));
+                            best = v > best ? v : best;
+                        }
                     }
-                }
             }
         }
 #pragma unroll
@@ -252,7 +270,7 @@ extern "C" bfm_status bfm_lambda(double alpha, double h, double T, int G, int re
     P.sd = (uint64_t)std::ldexp(std::sqrt(2.0 / (double)G), 63);
     P.h = h < 1.0 ? (uint64_t)std::ldexp(h, 64) : 0ull;
     P.stats = d_stats;
-    const int64_t slots = ((int64_t)ih + 63) / 32 * 32;
+    const int64_t slots = ((int64_t)ih + 2 * kSteps - 1) / kSteps * kSteps;
     const bool ring = (size_t)slots * kWarps * 8 <= kMaxRingBytes;
     P.ring = ring ? (int)slots : 0;
     e = ring ? launch_paths<true>(P, (size_t)slots * kWarps * 8, st) : launch_paths<false>(P, 0, st);
