@@ -624,7 +624,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
                 const HybridParams& Q = kBatch ? Bt.tiles[ti].P : P;
                 const int n = Q.n, N = Q.N;
-                const int nst = (n + G - 1) / G, per_block = 2 * nst + (N + G - 1) / G;
+                const int nsh = (n + G - 1) / G, per_block = 2 * nsh + (N + G - 1) / G;
                 if (px0 >= Q.m) {
                     pos0 += per_block;
                     s_pos[g] = pos0;
@@ -639,14 +639,14 @@ __global__ void __launch_bounds__(kThreads, 1)
                         ok = false;
                         break;
                     }
-                    ok = issue(tm, px0, d0, drop, pos0 + nst + d0 / G);
+                    ok = issue(tm, px0, d0, drop, pos0 + nsh + d0 / G);
                 }
                 if (!ok) break;
                 if (!wait_bar(coefb, 1u, abort_flag, kWaitNs)) {
                     raise_abort(abort_flag);
                     break;
                 }
-                for (int d0 = dstart(); d0 < N && ok; d0 += G) ok = issue(tm, px0, d0, normal, pos0 + 2 * nst + d0 / G);
+                for (int d0 = dstart(); d0 < N && ok; d0 += G) ok = issue(tm, px0, d0, normal, pos0 + 2 * nsh + d0 / G);
                 pos0 += per_block;
             }
             s_pos[g] = INT_MAX;

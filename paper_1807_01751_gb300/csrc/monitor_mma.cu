@@ -44,6 +44,7 @@
 #include <cmath>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 
 #include "bfm_internal.cuh"
 #include "ptx.cuh"
@@ -149,25 +150,6 @@ __device__ __forceinline__ void mma_xc(uint32_t dcol, uint32_t ccol, const unsig
     ptx::mma_f16_ta(dcol, ccol, bl, id, true);
 }
 
-template <typename T>
-struct YSmem;
-template <>
-struct YSmem<float> {
-    static __device__ __forceinline__ float get(const unsigned char* st, int idx, bool& valid) {
-        const float v = reinterpret_cast<const float*>(st)[idx];
-        valid = v == v;
-        return v;
-    }
-};
-template <>
-struct YSmem<int16_t> {
-    static __device__ __forceinline__ float get(const unsigned char* st, int idx, bool& valid) {
-        const int v = reinterpret_cast<const int16_t*>(st)[idx];
-        valid = v != -32768;
-        return (float)v;
-    }
-};
-
 __device__ __forceinline__ void tma_load_2d_hint(void* dst, const CUtensorMap* map, uint64_t* bar, int x, int y,
                                                  uint64_t pol) {
     asm volatile(
@@ -203,6 +185,7 @@ __device__ __forceinline__ void mma_block(const CUtensorMap* tmap, const MmaPara
     using B = Basis<KH>;
     constexpr int K = B::K, NBR = B::NBR;
     constexpr bool kInt = sizeof(T) == 2;
+    using Val = std::conditional_t<kInt, int, float>;
     constexpr int kStageBytes = kBlk * kTile * (int)sizeof(T);
     unsigned char* smem_raw = smem_base + kHdr;
     const size_t ta = (size_t)(P.npad / 8) * kTabLbo, tb = NBR > 16 ? (size_t)(P.nhpad / 8) * kTabLbo : 0;
@@ -281,83 +264,85 @@ __device__ __forceinline__ void mma_block(const CUtensorMap* tmap, const MmaPara
     // thread keeps S blocks in flight and refills a stage once its empty
     // barrier has seen kPairs arrivals (the producer's once a chunk is written in
     // the history passes, one from each first warp in the MOSUM pass).
-    uint32_t q_next = 0, s_q0 = 0;
-    int s_b0 = 0, s_b1 = 0, s_tlim = 0;
+    uint32_t q_next = 0;
+    int s_b1 = 0, s_tlim = 0;
     int producer = 0;  // thread 0 in the history passes, thread 128 in the MOSUM pass
     uint64_t s_pol = keep;
-    auto issue = [&](uint32_t q, int bd) {  // the producer thread
-        const int st = (int)(q % (uint32_t)S);
-        if (q >= (uint32_t)S) ok &= ptx::mbar_wait_bounded(empty + st, ((q / S) - 1u) & 1u, kWaitNs);
-        ptx::mbar_arrive_expect_tx(full + st, kStageBytes);
-        tma_load_2d_hint(sY + (size_t)st * kStageBytes, tmap, full + st, (int)p0, bd * kBlk, s_pol);
+    // The stage of the block at hand and of the next one to issue are counted along with
+    // their laps of the ring (a division per block and use took 5 % of the instructions).
+    int cslot = 0, pslot = 0, pblk = 0;
+    uint32_t clap = 0, plap = 0;
+    auto step = [&](int& slot, uint32_t& lap) {
+        ++slot;
+        lap += slot == S ? 1u : 0u;
+        slot = slot == S ? 0 : slot;
+    };
+    auto issue = [&]() {  // the producer thread: the next block of the pass
+        if (plap) ok &= ptx::mbar_wait_bounded(empty + pslot, (plap - 1u) & 1u, kWaitNs);
+        ptx::mbar_arrive_expect_tx(full + pslot, kStageBytes);
+        tma_load_2d_hint(sY + (size_t)pslot * kStageBytes, tmap, full + pslot, (int)p0, pblk * kBlk, s_pol);
+        ++pblk;
+        step(pslot, plap);
     };
     auto open = [&](int b0, int b1, int tlim, uint64_t pol) {
-        s_b0 = b0;
         s_b1 = b1;
-        s_q0 = q_next;
-        q_next += (uint32_t)(b1 - b0);
         s_pol = pol;
         s_tlim = tlim;
+        cslot = pslot = (int)(q_next % (uint32_t)S);
+        clap = plap = q_next / (uint32_t)S;
+        pblk = b0;
+        q_next += (uint32_t)(b1 - b0);
         if (tid == producer)
-            for (int j = 0; j < S && b0 + j < b1; ++j) issue(s_q0 + (uint32_t)j, b0 + j);
+            for (int j = 0; j < S && pblk < b1; ++j) issue();
     };
-    // the stage of date block bd, waited for
-    auto block_wait = [&](int bd) -> const unsigned char* {
-        const uint32_t q = s_q0 + (uint32_t)(bd - s_b0);
-        const int st = (int)(q % (uint32_t)S);
-        ok &= ptx::mbar_wait_bounded(full + st, (q / S) & 1u, kWaitNs);
-        return sY + (size_t)st * kStageBytes;
+    // the stage of the block at hand, waited for
+    auto block_wait = [&]() -> const unsigned char* {
+        ok &= ptx::mbar_wait_bounded(full + cslot, clap & 1u, kWaitNs);
+        return sY + (size_t)cslot * kStageBytes;
     };
-    // done with block bd: `count` arrivals (the producer refills the stage later)
-    auto block_release = [&](int bd, uint32_t count) {
-        const uint32_t q = s_q0 + (uint32_t)(bd - s_b0);
-        mbar_arrive_cnt(empty + (int)(q % (uint32_t)S), count);
+    // done with the block at hand: `count` arrivals (the producer refills the stage later)
+    auto block_release = [&](uint32_t count) { mbar_arrive_cnt(empty + cslot, count); };
+    auto block_next = [&]() { step(cslot, clap); };
+    auto block_refill = [&]() {  // the producer thread
+        if (pblk < s_b1) issue();
     };
-    auto block_refill = [&](int bd) {  // the producer thread
-        const uint32_t q = s_q0 + (uint32_t)(bd - s_b0);
-        if (bd + S < s_b1) issue(q + (uint32_t)S, bd + S);
+    // dates [t0, t0 + 8) of this pixel from a waited stage: values (0 where invalid; int16
+    // storage keeps integers) and validity (missing, masked, t >= tlim).  mbits: the pixel's
+    // mask bits of these dates.  Lanes past m see the zeros of the box's fill as data:
+    // nothing of theirs is written and nothing in them depends on the data's range.
+    auto read8 = [&](const unsigned char* sb, int t0, uint32_t mbits, Val (&y)[8], bool (&ok)[8]) {
+        const T* q = reinterpret_cast<const T*>(sb) + (t0 & (kBlk - 1)) * kTile + px;
+        auto get = [&](auto full_c) {
+            constexpr bool full = decltype(full_c)::value;  // every date is below tlim
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const Val v = (Val)q[e * kTile];
+                if constexpr (kInt)
+                    ok[e] = v != -32768;
+                else
+                    ok[e] = v == v;
+                if (!full) ok[e] = ok[e] && t0 + e < s_tlim;
+                if (kMask) ok[e] = ok[e] && ((mbits >> e) & 1u);
+                y[e] = ok[e] ? v : (Val)0;
+            }
+        };
+        if (t0 + 8 <= s_tlim)
+            get(std::true_type{});
+        else
+            get(std::false_type{});
     };
-    // dates [t0, t0 + 8) of this pixel from a waited stage: values (0 where
-    // invalid) and valid bits (missing, masked, t >= tlim, pixel beyond m);
-    // mbits: the pixel's mask bits of these dates
-    auto read8 = [&](const unsigned char* sb, int t0, uint32_t mbits, float (&y)[8]) -> uint32_t {
-        const int r0 = t0 & (kBlk - 1);
-        const int nt = s_tlim - t0;  // dates of the group before tlim
-        const uint32_t lim = !active || nt <= 0 ? 0u : (nt >= 8 ? 0xffu : (1u << nt) - 1u);
+    auto valid_bits = [](const bool (&ok)[8]) -> uint32_t {
         uint32_t vb = 0u;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            bool v;
-            y[e] = YSmem<T>::get(sb, (r0 + e) * kTile + px, v);
-            vb |= (v ? 1u : 0u) << e;
-        }
-        vb &= lim;
-        if constexpr (kMask) vb &= mbits;
-#pragma unroll
-        for (int e = 0; e < 8; ++e) y[e] = ((vb >> e) & 1u) ? y[e] : 0.f;
+        for (int e = 0; e < 8; ++e) vb |= ok[e] ? 1u << e : 0u;
         return vb;
     };
-    // the same as integers (int16 storage)
-    auto read8i = [&](const unsigned char* sb, int t0, uint32_t mbits, int (&y)[8]) -> uint32_t {
-        const int r0 = t0 & (kBlk - 1);
-        const int nt = s_tlim - t0;
-        uint32_t vb = !active || nt <= 0 ? 0u : (nt >= 8 ? 0xffu : (1u << nt) - 1u);
-        if constexpr (kMask) vb &= mbits;
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const int v = reinterpret_cast<const int16_t*>(sb)[(r0 + e) * kTile + px];
-            const bool ok = v != -32768 && ((vb >> e) & 1u);
-            y[e] = ok ? v : 0;
-            vb = ok ? vb : vb & ~(1u << e);
-        }
-        return vb;
-    };
-    // history passes: when a chunk is written every thread is done with block
-    // c, so thread 0 completes its empty phase at once and refills it
-    auto chunk_release = [&](int bd) {
+    // history passes: when a chunk is written every thread is done with its
+    // block, so thread 0 completes its empty phase at once and refills it
+    auto chunk_release = [&]() {
         if (tid == producer) {
-            block_release(bd, kPairs);
-            block_refill(bd);
+            block_release(kPairs);
+            block_refill();
         }
     };
 
@@ -365,7 +350,7 @@ __device__ __forceinline__ void mma_block(const CUtensorMap* tmap, const MmaPara
     // A buffer `buf` of chunk c is written: every warp says so and goes on, thread 0 waits
     // for all of them (which are then also done with Y block c) before it issues the
     // chunk's MMAs.  A CTA barrier per chunk cost 1.7 stall cycles per instruction here.
-    auto chunk_written = [&](int c, int buf) {
+    auto chunk_written = [&](int buf) {
         ptx::fence_async_smem();
         ptx::tc_fence_before();
         __syncwarp();
@@ -373,8 +358,9 @@ __device__ __forceinline__ void mma_block(const CUtensorMap* tmap, const MmaPara
         if (tid == 0) {
             ok &= ptx::mbar_wait_bounded(afull + buf, buf_uses[buf] & 1u, kWaitNs);
             ptx::tc_fence_after();
-            chunk_release(c);
+            chunk_release();
         }
+        block_next();
     };
     auto wait_done = [&]() {
         ok &= ptx::mbar_wait_bounded(bar_done, done_uses & 1u, kWaitNs);
@@ -415,34 +401,34 @@ __device__ __forceinline__ void mma_block(const CUtensorMap* tmap, const MmaPara
             const uint32_t mk16 = mb.cur >> ((c & 1) * kBlk);  // the chunk's mask bits
             unsigned char* pl = sA + (size_t)buf * kBufBytes;
             acquire(buf);
-            const unsigned char* sb = block_wait(c);
-            float yc[8];
-            if (!s_set) {  // float: the first group with a valid value sets s_y (earlier rows are 0)
+            const unsigned char* sb = block_wait();
+            if constexpr (!kInt)
+                if (!s_set) {  // the first group with a valid value sets s_y (earlier rows are 0)
 #pragma unroll
-                for (int g = 0; g < 2; ++g) {
-                    float yg[8];
-                    read8(sb, c * kBlk + g * 8, mk16 >> (g * 8), yg);
-                    float gm = 0.f;
+                    for (int g = 0; g < 2; ++g) {
+                        Val yg[8];
+                        bool okg[8];
+                        read8(sb, c * kBlk + g * 8, mk16 >> (g * 8), yg, okg);
+                        float gm = 0.f;
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) gm = fmaxf(gm, fabsf(yg[e]));
-                    if (!s_set && gm > 0.f) {
-                        s_y = pow2_scale(gm, 4);
-                        s_set = true;
+                        for (int e = 0; e < 8; ++e) gm = fmaxf(gm, fabsf(yg[e]));
+                        if (!s_set && gm > 0.f) {
+                            s_y = pow2_scale(gm, 4);
+                            s_set = true;
+                        }
                     }
                 }
-            }
-            int yi[8];
-            const uint32_t vc = kInt ? read8i(sb, c * kBlk + half * 8, mk16 >> (half * 8), yi)
-                                     : read8(sb, c * kBlk + half * 8, mk16 >> (half * 8), yc);
+            Val yc[8];
+            bool ok8[8];
+            read8(sb, c * kBlk + half * 8, mk16 >> (half * 8), yc, ok8);
             float mk[8], a1[8], a2[8];
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
-                const bool v = (vc >> e) & 1u;
-                mk[e] = v ? 1.f : 0.f;
+                mk[e] = ok8[e] ? 1.f : 0.f;
                 if constexpr (kInt) {
-                    yim = max(yim, abs(yi[e]));
-                    a1[e] = (float)(yi[e] & ~255);
-                    a2[e] = (float)(yi[e] & 255);
+                    yim = max(yim, abs(yc[e]));
+                    a1[e] = (float)(yc[e] & ~255);
+                    a2[e] = (float)(yc[e] & 255);
                 } else {
                     ym = fmaxf(ym, fabsf(yc[e]));
                     split_hi_lo(yc[e] * s_y, a1[e], a2[e]);
@@ -451,7 +437,7 @@ __device__ __forceinline__ void mma_block(const CUtensorMap* tmap, const MmaPara
             st_a(pl, px, half, mk);
             st_a(pl + kPlane, px, half, a1);
             st_a(pl + 2 * kPlane, px, half, a2);
-            chunk_written(c, buf);
+            chunk_written(buf);
             if (tid == 0) {
                 const int d0 = c * kBlk;
                 const bool first = c == 0;
@@ -560,10 +546,12 @@ __device__ __forceinline__ void mma_block(const CUtensorMap* tmap, const MmaPara
             const int t0 = c * kBlk + half * 8;
             unsigned char* pl = sA + (size_t)buf * kBufBytes;
             acquire(buf);
-            float yc[8], yh[8];
-            const unsigned char* sb = block_wait(c);
+            Val yc[8];
+            bool ok8[8];
+            float yh[8];
+            const unsigned char* sb = block_wait();
             if (kMask && !(c & 1)) mb.next(c * kBlk, lane);
-            const uint32_t vc = read8(sb, t0, mb.cur >> ((c & 1) * kBlk + half * 8), yc);
+            read8(sb, t0, mb.cur >> ((c & 1) * kBlk + half * 8), yc, ok8);
             ptx::tmem_wait_ld8(rq);
 #pragma unroll
             for (int e = 0; e < 8; ++e) yh[e] = __uint_as_float(rq[e]);
@@ -571,15 +559,14 @@ __device__ __forceinline__ void mma_block(const CUtensorMap* tmap, const MmaPara
             float rh[8], rl[8];
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
-                const bool v = (vc >> e) & 1u;
-                const float r0 = v ? (yc[e] - yh[e] * inv_b) : 0.f;
+                const float r0 = ok8[e] ? ((float)yc[e] - yh[e] * inv_b) : 0.f;
                 ss = fmaf(r0, r0, ss);
                 split_hi_lo(r0 * s_r, rh[e], rl[e]);
             }
-            sVb[(c * 2 + half) * kTile + px] = (unsigned char)vc;
+            sVb[(c * 2 + half) * kTile + px] = (unsigned char)valid_bits(ok8);
             st_a(pl, px, half, rh);
             st_a(pl + kPlane, px, half, rl);
-            chunk_written(c, buf);
+            chunk_written(buf);
             if (tid == 0) {
                 const int dd = c * kBlk;
                 const bool first = c == 0;
@@ -691,14 +678,16 @@ __device__ __forceinline__ void mma_block(const CUtensorMap* tmap, const MmaPara
             const unsigned char* sb = nullptr;
 #pragma unroll 1
             for (int c0 = d0; c0 < dend; c0 += 8, ++grp) {
-                float yc[8], yh[8];
-                const int bd = c0 / kBlk;
-                if ((c0 & 8) == 0) sb = block_wait(bd);
+                Val yc[8];
+                bool ok8[8];
+                float yh[8];
+                if ((c0 & 8) == 0) sb = block_wait();
                 if (kMask && !((c0 - d_start) & 31)) mb.next(c0, lane);
-                const uint32_t vb = read8(sb, c0, mb.cur >> ((c0 - d_start) & 31), yc);
+                read8(sb, c0, mb.cur >> ((c0 - d_start) & 31), yc, ok8);
                 if (c0 & 8) {
                     __syncwarp();
-                    if (lane == 0) block_release(bd, 1);
+                    if (lane == 0) block_release(1);
+                    block_next();
                 }
                 ptx::tmem_wait_ld8(rq);
 #pragma unroll
@@ -708,7 +697,7 @@ __device__ __forceinline__ void mma_block(const CUtensorMap* tmap, const MmaPara
                 float acc = 0.f;
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
-                    acc += ((vb >> e) & 1u) ? (yc[e] - yh[e] * inv_b) : 0.f;
+                    acc += ok8[e] ? ((float)yc[e] - yh[e] * inv_b) : 0.f;
                     loc[e] = acc;
                 }
                 // the base is the unevaluated sum Sh + Sc: each S is rounded once
@@ -724,25 +713,28 @@ __device__ __forceinline__ void mma_block(const CUtensorMap* tmap, const MmaPara
                 }
                 if (grp >= 2) ok &= ptx::mbar_wait_bounded(cons + (grp & 1), ((grp >> 1) - 1u) & 1u, kWaitNs);
                 // the slots are counted along (a popcount per date issues at an eighth of the rate)
+                const uint32_t vb = valid_bits(ok8);
                 mbox[(grp & 1) * kTile + px] = ((uint32_t)slot << 8) | vb;
+                float* wp = ring + slot * kTile + px;
                 if (slot <= R - 8) {  // the group's slots do not wrap
-                    float* wp = ring + slot * kTile + px;
 #pragma unroll
                     for (int e = 0; e < 8; ++e)
-                        if ((vb >> e) & 1u) {
+                        if (ok8[e]) {
                             *wp = Sv[e];
                             wp += kTile;
-                            ++slot;
                         }
-                    slot -= slot >= R ? R : 0;
                 } else {
+                    float* const end = ring + R * kTile + px;
 #pragma unroll
                     for (int e = 0; e < 8; ++e)
-                        if ((vb >> e) & 1u) {
-                            ring[slot * kTile + px] = Sv[e];
-                            slot = slot + 1 == R ? 0 : slot + 1;
+                        if (ok8[e]) {
+                            *wp = Sv[e];
+                            wp += kTile;
+                            wp = wp == end ? ring + px : wp;
                         }
                 }
+                slot += __popc(vb);
+                slot -= slot >= R ? R : 0;
                 __syncwarp();
                 if (lane == 0) mbar_arrive(rdy + (grp & 1));
             }
@@ -756,44 +748,47 @@ __device__ __forceinline__ void mma_block(const CUtensorMap* tmap, const MmaPara
                     const uint32_t word = mbox[(grp & 1) * kTile + px];
                     const uint32_t vb = word & 0xffu, mv = vb & mon;
                     const int sl0 = (int)(word >> 8);
-                    float wv[8], mo2[8];
-                    // slot of the next valid date and the slot h behind it, both in [0, R) (at an
-                    // invalid date they may hold anything: nothing of it is used)
-                    int se = sl0, ls = sl0 - h;
-                    ls += ls < 0 ? R : 0;
+                    // slot of the next valid date and the slot h behind it, both in [0, R), as
+                    // offsets into the pixel's column (at an invalid date they may hold anything:
+                    // nothing of it is used)
+                    const int end = R * kTile;
+                    int se = sl0 * kTile, ls = (sl0 - h) * kTile;
+                    ls += ls < 0 ? end : 0;
+                    const float* const col = ring + px;
+                    float wv[8], wm = 0.f;
 #pragma unroll
                     for (int e = 0; e < 8; ++e) {
-                        const float W = ring[se * kTile + px] - ring[ls * kTile + px];
-                        const float mo = W * inv_scale;
-                        const bool mm = (mv >> e) & 1u;
-                        wv[e] = mm ? W : 0.f;
-                        mo2[e] = mm ? mo * mo : 0.f;
+                        const float W = col[se] - col[ls];
+                        wv[e] = ((mv >> e) & 1u) ? W : 0.f;
+                        wm = fmaxf(wm, fabsf(wv[e]));
                         if ((vb >> e) & 1u) {
-                            se = se + 1 == R ? 0 : se + 1;
-                            ls = ls + 1 == R ? 0 : ls + 1;
+                            se = se + kTile == end ? 0 : se + kTile;
+                            ls = ls + kTile == end ? 0 : ls + kTile;
                         }
                     }
-                    // log+ >= 1: |MO| <= lambda never crosses; the exact boundary
-                    // only for candidates before the first crossing
-                    uint32_t cand = 0u;
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) cand |= (mo2[e] > lam2 ? 1u : 0u) << e;
-                    if (brk < 0 && cand) {
+                    // log+ >= 1: |MO| <= lambda never crosses; the exact boundary only for
+                    // candidates before the first crossing (rounding is monotonic, so the
+                    // largest |W| has the largest MO^2 of the group)
+                    const float mm = wm * inv_scale;
+                    if (brk < 0 && mm * mm > lam2) {
                         int jb = jm;
 #pragma unroll
                         for (int e = 0; e < 8; ++e) {
-                            if (brk < 0 && ((cand >> e) & 1u)) {
+                            const float mo = wv[e] * inv_scale, mo2 = mo * mo;
+                            if (brk < 0 && ((mv >> e) & 1u) && mo2 > lam2) {
                                 const int J = n_i + jb + 1;
                                 const float b2 = J > jlim ? lam2 * kLn2f * (log2_fast((float)J) - lg_n) : lam2;
-                                if (mo2[e] > b2) brk = c0 + e;
+                                if (mo2 > b2) brk = c0 + e;
                             }
                             jb += (mv >> e) & 1u;
                         }
                     }
                     if (want_mx) {
 #pragma unroll
-                        for (int e = 0; e < 8; ++e)
-                            if (((mv >> e) & 1u) && mo2[e] > mx * mx) mx = wv[e] * inv_scale;
+                        for (int e = 0; e < 8; ++e) {
+                            const float mo = wv[e] * inv_scale;
+                            if (((mv >> e) & 1u) && mo * mo > mx * mx) mx = mo;
+                        }
                     }
                     jm += __popc(mv);
                     // the group's windows summed as a tree, then one compensated add
@@ -802,7 +797,7 @@ __device__ __forceinline__ void mma_block(const CUtensorMap* tmap, const MmaPara
                 }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(cons + (grp & 1));
-                if (tid == producer && (c0 & 8)) block_refill(c0 / kBlk);
+                if (tid == producer && (c0 & 8)) block_refill();
             }
         }
     }
@@ -893,7 +888,7 @@ constexpr size_t kSmemTwo = 115712;  // shared memory per CTA with two CTAs on a
 // or 6 (int16) stages, or as few as 2 (float) or 4 (int16) where that lets two CTAs
 // share an SM.  On 1.95 Mi int16 pixels of 586 dates (history 347, ring of 103 slots, 116 KB
 // with six stages and 112 with five) two CTAs took 5.03 ms, one 8.50; with the chunk and
-// group hand-offs per warp and the ring slots counted along, 4.85.
+// group hand-offs per warp and ring and stage slots counted along, 4.49.
 MmaLayout mma_layout(int npad, int nhpad, int k, int ring, int elt) {
     MmaLayout L{};
     const size_t ta = (size_t)(npad / 8) * kTabLbo;
