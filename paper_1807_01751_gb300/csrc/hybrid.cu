@@ -92,7 +92,8 @@ constexpr int kStages = 3;                // stages in flight per group
 // With all four M-tiles in one group the kernel issued on 58 % of its cycles, with two
 // groups 68 %: 7.50 -> 6.70 ms (float) and 7.63 -> 6.91 ms (int16) on 8.4 Mi pixels of 414
 // dates, 193 -> 167 us on 250k pixels of 256; with whole chunks and groups in loops of
-// their own, without bounds checks, 6.48 ms, 6.49 ms and 154 us.  One M-tile per group (24 warps, 80
+// their own, without bounds checks, 6.48 ms, 6.49 ms and 154 us, and with the ring
+// addressed directly 6.30, 6.41 and 154.  One M-tile per group (24 warps, 80
 // registers) was slower at every size but the smallest.
 constexpr int kGrp = 2;                       // M-tiles per group
 constexpr int kGroups = kMT / kGrp;
@@ -377,11 +378,22 @@ __device__ __forceinline__ void pass_b8(const Obs<T, kMask>& ob, const T (&raw)[
     }
 }
 
+// The ring is addressed by 32-bit shared-memory addresses, so that a slot needs no
+// address arithmetic of its own.
+__device__ __forceinline__ float ring_ld(uint32_t a) {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ void ring_st(uint32_t a, float v) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v)); }
+constexpr uint32_t kSlot = kPx * 4;  // bytes from slot to slot
+
 // State of the monitoring scan of one pixel.
 struct Mon {
-    int slot = 0;         // ring slot (float offset) of the next residual
-    int hp_off = 0;       // h_p slots
-    int fill_end = 0;     // h_p - 1 slots: the first window's history part
+    uint32_t slot = 0;    // address of the next residual's ring slot
+    uint32_t beg = 0;     // of the first slot
+    uint32_t end = 0;     // behind h_p slots
+    uint32_t fill_end = 0;  // behind h_p - 1 slots: the first window's history part
     int wdate = 0;        // date of the first window's oldest history observation
     int cnt = 0;          // valid monitoring observations so far
     float inv_sb = 1.f;
@@ -394,27 +406,26 @@ struct Mon {
 // History dates [d8, d8 + 8) before n: the first window's residuals into the ring.
 template <typename T, bool kMask>
 __device__ __forceinline__ void mon_hist8(const Obs<T, kMask>& ob, const T (&raw)[8], int d8, const float* yh,
-                                          float* ring_t, Mon& mo) {
+                                          Mon& mo) {
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
         bool ok;
         const float y = ob.value(raw[u], u, true, ok);
         const float r = fmaf(-yh[u], mo.inv_sb, y);
         const bool take = ok && d8 + u >= mo.wdate && mo.slot < mo.fill_end;
-        if (take) ring_t[mo.slot] = r;
-        mo.slot += take ? kPx : 0;
+        if (take) ring_st(mo.slot, r);
+        mo.slot += take ? kSlot : 0u;
         mo.W += take ? r : 0.f;
     }
 }
 
 // One monitoring date: the window gains r and loses the ring slot it replaces.
 template <bool kExt>
-__device__ __forceinline__ void mon_step(bool ok, float r, float* ring_t, Mon& mo) {
-    float* a = ring_t + mo.slot;
-    const float old = *a;
-    if (ok) *a = r;
-    const int ns = mo.slot + (ok ? kPx : 0);
-    mo.slot = ns == mo.hp_off ? 0 : ns;
+__device__ __forceinline__ void mon_step(bool ok, float r, Mon& mo) {
+    const float old = ring_ld(mo.slot);
+    if (ok) ring_st(mo.slot, r);
+    const uint32_t ns = mo.slot + (ok ? kSlot : 0u);
+    mo.slot = ns == mo.end ? mo.beg : ns;
     mo.W += ok ? r - old : 0.f;
     mo.cnt += ok ? 1 : 0;
     mo.blk += ok ? mo.W : 0.f;
@@ -427,13 +438,13 @@ __device__ __forceinline__ void mon_step(bool ok, float r, float* ring_t, Mon& m
 
 // Eight monitoring dates, all in [n, N).
 template <bool kExt, typename T, bool kMask>
-__device__ __forceinline__ void mon8(const Obs<T, kMask>& ob, const T (&raw)[8], const float* yh, float* ring_t,
-                                     Mon& mo, float (&Wu)[8]) {
+__device__ __forceinline__ void mon8(const Obs<T, kMask>& ob, const T (&raw)[8], const float* yh, Mon& mo,
+                                     float (&Wu)[8]) {
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
         bool ok;
         const float y = ob.value(raw[u], u, true, ok);
-        mon_step<kExt>(ok, fmaf(-yh[u], mo.inv_sb, y), ring_t, mo);
+        mon_step<kExt>(ok, fmaf(-yh[u], mo.inv_sb, y), mo);
         Wu[u] = mo.W;
     }
 }
@@ -441,7 +452,7 @@ __device__ __forceinline__ void mon8(const Obs<T, kMask>& ob, const T (&raw)[8],
 // Dates [d8, d8 + 8) that hold n (or N): history dates fill the ring, later ones are monitored.
 template <typename T, bool kMask>
 __device__ __forceinline__ void mon_mixed8(const Obs<T, kMask>& ob, const T (&raw)[8], int d8, int n, int N,
-                                        const float* yh, float* ring_t, Mon& mo, float (&Wu)[8], bool ext) {
+                                        const float* yh, Mon& mo, float (&Wu)[8], bool ext) {
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
         const int d = d8 + u;
@@ -450,13 +461,13 @@ __device__ __forceinline__ void mon_mixed8(const Obs<T, kMask>& ob, const T (&ra
         const float r = fmaf(-yh[u], mo.inv_sb, y);
         if (d < n) {
             const bool take = ok && d >= mo.wdate && mo.slot < mo.fill_end;
-            if (take) ring_t[mo.slot] = r;
-            mo.slot += take ? kPx : 0;
+            if (take) ring_st(mo.slot, r);
+            mo.slot += take ? kSlot : 0u;
             mo.W += take ? r : 0.f;
         } else if (ext) {
-            mon_step<true>(ok, r, ring_t, mo);
+            mon_step<true>(ok, r, mo);
         } else {
-            mon_step<false>(ok, r, ring_t, mo);
+            mon_step<false>(ok, r, mo);
         }
         Wu[u] = mo.W;
     }
@@ -803,7 +814,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint32_t tl = (uint32_t)(32 * q) << 16;       // TMEM lane field of this warp
         const uint32_t tcol = tmem + 128u * (uint32_t)(w >> 2);  // this M-tile's columns
         const int gp = pl % kGrpPx;                         // pixel within the group's block
-        float* ring_t = ring + pl;
+        const uint32_t ring_a = ptx::smem_u32(ring + pl);
         const T* sbase =
             reinterpret_cast<const T*>(stages + g * (kStages * kStageBytes) + (gp >> 7) * kBoxBytes) + (pl & 127);
         const float qnan = __int_as_float(0x7fc00000);
@@ -1148,11 +1159,12 @@ __global__ void __launch_bounds__(kThreads, 1)
             float* const maxmo = Q.maxmo;
             const float jlimf = (float)floor(kEuler * (double)np);  // J / n_p <= e  <=>  J <= jlim
             Mon mo{};
-            mo.hp_off = hp * kPx;
-            mo.fill_end = (hp - 1) * kPx;
+            mo.beg = mo.slot = ring_a;
+            mo.end = ring_a + (uint32_t)hp * kSlot;
+            mo.fill_end = mo.end - kSlot;
             mo.wdate = wdate;
             mo.inv_sb = inv_fit;
-            ring_t[(hp - 1) * kPx] = 0.f;  // the first monitoring step finds h_p - 1 residuals
+            ring_st(mo.fill_end, 0.f);  // the first monitoring step finds h_p - 1 residuals
             int brk = -1;
             float sh = 0.f, sl = 0.f;
             const T* stg = nullptr;
@@ -1213,7 +1225,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const int J0 = np + 1 + mo.cnt;
                 mo.blk = 0.f;
                 mo.amax = 0.f;
-                mon_mixed8(ob, raw, d8, n, N, yh, ring_t, mo, Wu, maxmo != nullptr);
+                mon_mixed8(ob, raw, d8, n, N, yh, mo, Wu, maxmo != nullptr);
                 test8(d8, J0, raw, Wu);
                 end8(d8);
                 return true;
@@ -1225,7 +1237,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const int J0 = np + 1 + mo.cnt;
                 mo.blk = 0.f;
                 mo.amax = 0.f;
-                mon8<decltype(ext_c)::value>(ob, raw, yh, ring_t, mo, Wu);
+                mon8<decltype(ext_c)::value>(ob, raw, yh, mo, Wu);
                 test8(d8, J0, raw, Wu);
                 end8(d8);
                 return true;
@@ -1235,7 +1247,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 T raw[8];
                 float yh[8];
                 if (!begin8(d8, raw, yh)) break;
-                mon_hist8(ob, raw, d8, yh, ring_t, mo);
+                mon_hist8(ob, raw, d8, yh, mo);
                 end8(d8);
             }
             if (d8 < n && !bad && mixed(d8)) d8 += 8;
