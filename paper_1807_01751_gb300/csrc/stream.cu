@@ -3,8 +3,8 @@
 //
 // Each pixel's column of Y is streamed four times through shared memory
 // (pass A, A', B over the history, pass C over the monitoring dates), in
-// stages filled by 2-D TMA boxes (256 pixels x 8 dates: three float or six
-// int16 stages) that a producer warp issues up to a full ring ahead; the history stays
+// stages filled by 2-D TMA boxes (256 pixels x 8 dates: three float, six
+// or three int16 stages) that a producer warp issues up to a full ring ahead; the history stays
 // in L2 between its passes (evict-last hints, a grid sized to the L2), so Y
 // is read once from DRAM.  Per pixel (Section 2.1, Eq. 3-6, Algorithm 1 with
 // missing values masked, as in the other forms):
@@ -88,6 +88,7 @@ constexpr double kL2Budget = 80e6;           // bytes of history the resident pi
 constexpr uint64_t kWaitNs = 2000000000ull;  // bound of every wait
 
 struct StreamParams {
+    int stages;        // stages in flight (int16)
     uint64_t wait_ns;  // bound of the consumers' stage waits (bfm_stage_wait_limit)
     const uint32_t* mask;
     int64_t m, mask_words;
@@ -119,6 +120,11 @@ __device__ __forceinline__ bool obs(int16_t raw, float& y) {
 struct Layout {
     size_t phi, xm, ring, stages, bars, total;
 };
+// With three harmonics and int16 storage the 21 basis sums wait for the second solve in the
+// ring, which is idle until pass B: in registers they make pass A' spill (500k pixels of 414
+// dates 654 us, 644 so with six stages fixed; float storage is the faster with its few spills, 9.24 ms against 9.34
+// on 8.4 Mi pixels).
+constexpr int kStashed = Basis<3>::NBR;
 
 __host__ __device__ inline size_t up128(size_t x) { return (x + 127) & ~(size_t)127; }
 
@@ -127,9 +133,12 @@ __host__ __device__ inline Layout stream_layout(int N, int n, int K, int NB, int
     L.phi = 0;
     L.xm = up128(sizeof(float) * (size_t)n * NB);
     L.ring = L.xm + up128(sizeof(float) * (size_t)(N - n) * K);
-    L.stages = L.ring + up128(sizeof(float) * (size_t)hmax * kThreads);
+    const int slots = K == 8 && hmax < kStashed ? kStashed : hmax;
+    L.stages = L.ring + up128(sizeof(float) * (size_t)slots * kThreads);
     L.bars = L.stages + (size_t)kStageArea;
-    L.total = L.bars + 2 * kMaxStages * sizeof(uint64_t) + 16;  // what decides whether a call takes this form
+    // what decides whether a call takes this form: the ring alone, and 112 bytes
+    L.total = L.bars - up128(sizeof(float) * (size_t)slots * kThreads) + up128(sizeof(float) * (size_t)hmax * kThreads) +
+              2 * kMaxStages * sizeof(uint64_t) + 16;
     return L;
 }
 
@@ -141,9 +150,10 @@ __global__ void __launch_bounds__(kThreads + 32, 2)
     stream_kernel(const __grid_constant__ CUtensorMap tmap, const StreamParams P) {
     using B = Basis<KH>;
     constexpr int K = B::K, NB = B::NB, NBR = B::NBR;
+    constexpr bool kStash = NBR == kStashed && sizeof(T) == 2;
     constexpr int G = kDates;                    // dates per stage
     constexpr int kStageBytes = Stage<T>::kBytes;
-    constexpr int kStages = Stage<T>::kCount;    // stages in flight
+    const int kStages = sizeof(T) == 4 ? Stage<T>::kCount : P.stages;  // stages in flight
     extern __shared__ __align__(128) unsigned char smem[];
     const int n = P.n, N = P.N, hmax = P.hmax;
     const int64_t m = P.m;
@@ -335,8 +345,10 @@ __global__ void __launch_bounds__(kThreads + 32, 2)
         for (; d0 + G <= n && !bad; d0 += G) passA(d0, std::true_type{});
         if (d0 < n && !bad) passA(d0, std::false_type{});
         const int np = (int)S[0];  // basis row 0 is 1: S[0] counts the valid history dates
-        int hp = (int)floor(P.h_frac * (double)np);
-        hp = hp < 1 ? 1 : (hp > np ? np : hp);
+        auto window = [&]() -> int {
+            const int h = (int)floor(P.h_frac * (double)np);
+            return h < 1 ? 1 : (h > np ? np : h);
+        };
         float b0[K];
         bool nonsingular;
         {
@@ -345,12 +357,18 @@ __global__ void __launch_bounds__(kThreads + 32, 2)
             nonsingular = cholesky<K>(Gm, Lc, dinv);
             chol_solve<K>(Lc, dinv, Bv, b0);
         }
+        if constexpr (kStash) {
+#pragma unroll
+            for (int i = 0; i < NBR; ++i) ring[i * kThreads] = S[i];
+        }
 
         const bool fit = np > K && nonsingular;
 
         // pass A': residuals r0 of the first solution, refinement sums c = X'M r0, and the
-        // date of the window's oldest history observation (0-based valid rank n_p - h_p + 1)
-        int rem = fit ? np - hp + 1 : np, wdate = n;
+        // date of the window's oldest history observation (0-based valid rank n_p - h_p + 1).
+        // rem: the valid history observations before that one; ~date once it is found (one
+        // register, which this pass has few of).
+        int rem = fit ? np - window() + 1 : np;
         float cr[K];
 #pragma unroll
         for (int a = 0; a < K; ++a) cr[a] = 0.f;
@@ -359,6 +377,7 @@ __global__ void __launch_bounds__(kThreads + 32, 2)
             constexpr bool full = decltype(full_c)::value;
             constexpr bool scan = decltype(scan_c)::value;  // a pixel of the warp may reach its window
             const int cnt = full ? G : n - d0;
+            const int left = rem >= 0 ? 1 : 0;
 #pragma unroll
             for (int u = 0; u < G; ++u) {
                 float y;
@@ -368,8 +387,10 @@ __global__ void __launch_bounds__(kThreads + 32, 2)
                 ss0 = fmaf(r, r, ss0);
 #pragma unroll
                 for (int a = 0; a < K; ++a) cr[a] = fmaf(ph[a], r, cr[a]);
-                if (scan) wdate = v != 0.f && rem == 0 ? d0 + u : wdate;
-                rem -= v != 0.f ? 1 : 0;
+                if (scan)
+                    rem = v != 0.f && rem >= 0 ? (rem == 0 ? ~(d0 + u) : rem - 1) : rem;
+                else
+                    rem -= v != 0.f ? left : 0;
             }
         };
         if (kMask) mb.open(0, lane);
@@ -378,12 +399,13 @@ __global__ void __launch_bounds__(kThreads + 32, 2)
             const uint32_t bits = mask_bits(d0, 0);
             if (d0 + G > n)
                 passA2(d0, std::false_type{}, std::true_type{}, st, bits);
-            else if (__any_sync(~0u, rem < G))
+            else if (__any_sync(~0u, (unsigned)rem < (unsigned)G))
                 passA2(d0, std::true_type{}, std::true_type{}, st, bits);
             else
                 passA2(d0, std::true_type{}, std::false_type{}, st, bits);
             release();
         }
+        const int wdate = rem < 0 ? ~rem : n;
         {
             const unsigned w = __reduce_min_sync(~0u, (unsigned)(active ? wdate : n));
             if ((threadIdx.x & 31) == 0) {
@@ -393,6 +415,10 @@ __global__ void __launch_bounds__(kThreads + 32, 2)
         }
         float dl[K];
         {
+            if constexpr (kStash) {
+#pragma unroll
+                for (int i = 0; i < NBR; ++i) S[i] = ring[i * kThreads];
+            }
             float Gm[K][K], Lc[K][K], dinv[K];
             gram_from_sums<KH>(S, Gm);
             cholesky<K>(Gm, Lc, dinv);
@@ -403,7 +429,7 @@ __global__ void __launch_bounds__(kThreads + 32, 2)
         for (int a = 0; a < K; ++a) dc = fmaf(dl[a], cr[a], dc);
         const float sig = sqrtf(fmaxf(ss0 - dc, 0.f) / (float)(np - K));
         const bool degenerate = !(sig > kDegenerateRatio * ymax) || ymax == 0.f;
-        if (!fit) hp = 1;  // keeps the ring arithmetic in range; nothing of it is used
+        const int hp = fit ? window() : 1;  // 1 keeps the ring arithmetic in range; nothing of it is used
         float bres[K];  // coefficients of the residuals: intercept and trend as hi (bres) + lo (dl)
 #pragma unroll
         for (int a = 0; a < K; ++a) bres[a] = a < 2 ? b0[a] : b0[a] + dl[a];
@@ -613,6 +639,11 @@ bfm_status launch_stream(const bfm_design_s* d, int dtype, const void* Y, const 
     }
     const size_t elt = dtype == BFM_F32 ? 4 : 2;
     StreamParams P{};
+    // int16 has room for six stages, but with rows of 16 MB the 96 dates that two CTAs then
+    // have in flight lie on more pages than the SM's address translations cover: 10.87 ms on
+    // 8.4 Mi pixels (K = 8), 9.77 with three.  At rows of 4 MB both take 2.36 ms on 2 Mi
+    // pixels, below that six are 1 % faster.
+    P.stages = (size_t)m * elt > ((size_t)4 << 20) ? 3 : Stage<int16_t>::kCount;
     P.wait_ns = stage_wait_ns();
     P.mask = mask;
     P.m = m;
