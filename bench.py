@@ -42,9 +42,9 @@ sys.path.insert(0, ROOT)
 METRIC = "BFAST-monitor pixels/s at 8.4M px x 414 dates; p50/p99 tile latency"
 # DRAM bytes per pixel per launch from the ncu captures summarised in
 # profiles/ (None once the kernel changes after the capture).
-TRAFFIC_PER_PX = {"f32": (1.7866e9 / 1048576,), "f32simt": (1.784346e9 / 1048576,), "f32stream": (None,),
-                  "i16": (None,), "f32hybrid": (1.836045e9 / 1048576,), "i16hybrid": (None,),
-                  "i16stream": (None,), "f32complete": (None,)}
+TRAFFIC_PER_PX = {"f32": (1.78515e9 / 1048576,), "f32simt": (1.78385e9 / 1048576,), "f32stream": (1.86174e9 / 1048576,),
+                  "i16": (0.911513e9 / 1048576,), "f32hybrid": (1.83945e9 / 1048576,), "i16hybrid": (0.914645e9 / 1048576,),
+                  "i16stream": (0.912723e9 / 1048576,), "f32complete": (1.82763e9 / 1048576,)}
 SAMPLE_PX = 4096  # pixels of each timed form checked against the oracle (outside the timed region)
 
 WORKLOAD = "c2: full scene 8,388,608 px x 414 dates, n_hist=228, K=8, f=23, h=0.25, plain float32"
@@ -600,7 +600,7 @@ def run_ours(args):
         lam_ms = (time.perf_counter() - t0) * 1e3
         lam_sim = {"alpha": 0.05, "h": 0.25, "T": N / n_hist, "grid_per_unit": 1000, "paths": 100000,
                    "lambda": lam_v, "ms": lam_ms, "paths_per_s": 1e5 / (lam_ms / 1e3),
-                   "note": "bfm_lambda, one FP64 path per thread, host quantile; wall time of the call"}
+                   "note": "bfm_lambda, one fixed-point path per warp, quantile on the device; wall time of the call"}
 
     # the per-pixel solve of Eq. 6 (two per pixel) in FP64 and in FP32, for every pixel of the scene
     solve = None

@@ -103,9 +103,9 @@ enum {
  * coefficients and regressors) per 32-date piece, and the refinement sums
  * X'M r0 (fp16 hi + lo residuals).  512 pixels per CTA, one CTA per SM, three
  * passes over each pixel's column (history twice, then the dates from the
- * earliest first-window observation of the tile on).  Same outputs and
+ * earliest first-window observation of a block of 256 pixels on).  Same outputs and
  * conventions as BFM_ALGO_STREAM.  Needs Y with a 16-byte aligned base and
- * rows of a multiple of 16 bytes, and the tables, three 16 KB stages and a
+ * rows of a multiple of 16 bytes, and the tables, 48 KB of stages and a
  * ring of floor(h_frac * n_hist) residuals for 512 pixels within one SM's
  * shared memory (else BFM_EUNSUPPORTED). */
 typedef enum {
