@@ -1,6 +1,5 @@
 // C ABI of libbfm: argument checks, the design cache, dispatch to the
 // kernels, and the host-buffer entry point (chunked copy/compute overlap).
-#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -53,6 +52,27 @@ void basis_rows(const bfm_design_s& d, std::vector<double>& rows) {
                 r[TS(j)] = tp * sj;
                 r[TS(j) + 1] = tp * cj;
             }
+        }
+    }
+}
+
+// The regressors of Eq. 2 in FP64 for bfm_trace [N][K].  sin and cos of pi x, x = 2 j t / f,
+// after folding x exactly to a quarter turn around 0: their error is that of x alone.  (The
+// rows above multiply by 2 pi first, which costs up to 5e-12 for dates in decimal years;
+// that is far below the float and fp16 tables made of them, but not below bfm_trace.)
+void trace_rows(const bfm_design_s& d, std::vector<double>& rows) {
+    rows.resize((size_t)d.N * d.K);
+    for (int t = 0; t < d.N; ++t) {
+        double* r = rows.data() + (size_t)t * d.K;
+        r[0] = 1.0;
+        r[1] = (d.dates[t] - d.c) / d.s;
+        for (int j = 1; j <= d.k; ++j) {
+            const double x = std::fmod(2.0 * (double)j * d.dates[t] / d.f, 2.0);  // exact
+            const double q = std::nearbyint(2.0 * x);                             // quarter turns
+            const double a = 3.14159265358979323846 * (x - 0.5 * q), s = std::sin(a), c = std::cos(a);
+            const int turn = (int)q & 3;
+            r[2 * j] = turn == 0 ? s : turn == 1 ? c : turn == 2 ? -s : -c;
+            r[2 * j + 1] = turn == 0 ? c : turn == 1 ? -s : turn == 2 ? -c : s;
         }
     }
 }
@@ -286,8 +306,8 @@ bfm_status bfm_design_create(const double* dates, int N, int k_harm, double f, b
         if (e == cudaSuccess) e = cudaMemcpy(d->d_hyb, tab.data(), tab.size(), cudaMemcpyHostToDevice);
     }
     if (e == cudaSuccess) {
-        std::vector<double> x((size_t)N * d->K);  // the first K entries of every basis row
-        for (int t = 0; t < N; ++t) std::copy_n(rowsd.begin() + (size_t)t * d->NB, d->K, x.begin() + (size_t)t * d->K);
+        std::vector<double> x;
+        trace_rows(*d, x);
         e = cudaMalloc(&d->d_xd, x.size() * sizeof(double));
         if (e == cudaSuccess) e = cudaMemcpy(d->d_xd, x.data(), x.size() * sizeof(double), cudaMemcpyHostToDevice);
     }
