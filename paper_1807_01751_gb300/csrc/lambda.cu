@@ -37,6 +37,8 @@
 namespace bfm {
 namespace {
 
+using fixedpt::Count;
+
 constexpr uint64_t kGolden = 0x9E3779B97F4A7C15ull;  // SplitMix64 increment
 constexpr int kWarps = 4;                             // paths at a time per block
 constexpr int kPer = 2;                               // consecutive steps of a lane
@@ -91,7 +93,7 @@ __global__ void __launch_bounds__(kSelThreads) kth_smallest(double* v, int n, in
         const int shift = top > kSelBits ? top - kSelBits : 0, width = top - shift;
         for (int i = threadIdx.x; i < (1 << kSelBits); i += kSelThreads) hist[i] = 0;
         __syncthreads();
-        for (int i = threadIdx.x; i < n; i += kSelThreads) {
+        for (Count i = threadIdx.x; i < (Count)n; i += kSelThreads) {
             const uint64_t u = (uint64_t)__double_as_longlong(v[i]);
             if (top == 64 || (u >> top) == (prefix >> top)) atomicAdd(&hist[(int)((u >> shift) & ((1u << width) - 1u))], 1);
         }
@@ -148,8 +150,8 @@ __global__ void __launch_bounds__(32 * kWarps)
             __syncwarp();  // the previous path's reads
             if (lane == 0) ring[P.ring - 1] = 0;  // W(0), the slot before step 1
         }
-        for (int i0 = 1; i0 <= P.nsteps; i0 += kSteps) {
-            const int i = i0 + kPer * lane;  // this lane's steps i, i + 1
+        for (Count i0 = 1; i0 <= (Count)P.nsteps; i0 += kSteps) {
+            const Count i = i0 + kPer * lane;  // this lane's steps i, i + 1
             int64_t W[kPer];
             {
                 const int64_t d0 = increment(st, P, s_ln, s_rec), d1 = increment(st + 2 * kGolden, P, s_ln, s_rec);
@@ -171,31 +173,31 @@ __global__ void __launch_bounds__(32 * kWarps)
                 pos += kSteps;
                 pos = pos == P.ring ? 0 : pos;
                 __syncwarp();
-            } else if (i0 + kSteps - 1 > P.ih) {
+            } else if (i0 + kSteps - 1 > (Count)P.ih) {
                 int64_t d[kPer];  // the lagged steps
 #pragma unroll
                 for (int u = 0; u < kPer; ++u) {
-                    const int j = i + u - P.ih;
+                    const int j = (int)(i + u - (Count)P.ih);
                     d[u] = j >= 1 ? increment(s0 + 2 * kGolden * (uint64_t)(j - 1), P, s_ln, s_rec) : 0;
                 }
                 lag[1] = lbase + warp_scan(d[0] + d[1], lane);
                 lag[0] = lag[1] - d[1];
                 lbase = __shfl_sync(~0u, lag[1], 31);
             }
-            if (i0 + kSteps - 1 >= P.G) {
-                if (i0 <= P.G) {  // W(1) is in this block
-                    const int at = P.G - i0;
+            if (i0 + kSteps - 1 >= (Count)P.G) {
+                if (i0 <= (Count)P.G) {  // W(1) is in this block
+                    const int at = (int)((Count)P.G - i0);
                     const int64_t w1 = __shfl_sync(~0u, (at & 1) ? W[1] : W[0], at >> 1);
                     const uint64_t a = (uint64_t)(w1 < 0 ? -w1 : w1), ha = P.h ? __umul64hi(a, P.h) : a;
                     hw1 = w1 < 0 ? -(int64_t)ha : (int64_t)ha;
                 }
 #pragma unroll
                 for (int u = 0; u < kPer; ++u)
-                    if (i + u >= P.G && i + u <= P.nsteps) {
+                    if (i + u >= (Count)P.G && i + u <= (Count)P.nsteps) {
                         const int64_t z = W[u] - lag[u] - hw1;
                         uint64_t v = (uint64_t)(z < 0 ? -z : z);
                         if (v > best) {  // the boundary's factor, at least 1, only lowers it
-                            if (i + u > P.ie) v = (uint64_t)((double)v / sqrt(log((double)(i + u) / (double)P.G)));
+                            if (i + u > (Count)P.ie) v = (uint64_t)((double)v / sqrt(log((double)(i + u) / (double)P.G)));
                             best = v > best ? v : best;
                         }
                     }

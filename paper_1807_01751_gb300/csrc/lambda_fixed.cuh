@@ -28,6 +28,10 @@
 namespace bfm {
 namespace fixedpt {
 
+// Counts of steps and paths go up to 2^31 - 1; a loop over them ends one stride later,
+// which 32 signed bits do not hold.
+typedef uint32_t Count;
+
 constexpr uint64_t kLn2Q64 = 0xB17217F7D1CF79ABull;  // ln 2 * 2^64
 
 // floor(a b / 2^64) or one less (the product of the low halves is dropped), for a and b
