@@ -3,10 +3,9 @@
 //
 // Each pixel's column of Y is streamed four times through shared memory
 // (pass A, A', B over the history, pass C over the monitoring dates), in
-// stages filled by 2-D TMA boxes (256 pixels x 8 dates: three float, six
-// or three int16 stages) that a producer warp issues up to a full ring ahead; the history stays
-// in L2 between its passes (evict-last hints, a grid sized to the L2), so Y
-// is read once from DRAM.  Per pixel (Section 2.1, Eq. 3-6, Algorithm 1 with
+// stages filled by 2-D TMA boxes (256 pixels x 8 dates) that a producer
+// warp issues up to a full ring ahead; the history stays in L2 between its
+// passes (evict-last hints, a grid sized to the L2), so Y is read once from DRAM.  Per pixel (Section 2.1, Eq. 3-6, Algorithm 1 with
 // missing values masked, as in the other forms):
 //   A   masked sums of the basis functions of bfm::Basis over the valid
 //       history dates -> Gram matrix G (identities of gram_from_sums) and
@@ -30,7 +29,8 @@
 //
 // Bound by instruction issue (75 % of the cycles).  Pass B from the window's start
 // instead of the history's, and the boundary only where a batch's largest |MO| can
-// reach it, took 500k int16 pixels of 522 dates (one harmonic) from 661 to 548 us.  Two
+// reach it, took 500k int16 pixels of 522 dates (one harmonic) from 661 to 555 us, a
+// boundary search without positions and the window starts from bits to 515.  Two
 // pixels per thread with f32x2 arithmetic issued a third fewer instructions, but the
 // ring leaves room for 512 pixels, so eight warps: 52 % issue, 627 us; not kept.
 #include <cudaTypedefs.h>
@@ -75,20 +75,32 @@ using namespace stage;
 
 constexpr int kThreads = 256;                // pixels per CTA (eight consumer warps)
 constexpr int kDates = 8;                    // dates per stage (one TMA box of 256 pixels x 8 dates)
-constexpr int kStageArea = 24576;            // bytes of stages per CTA: 3 float or 6 int16 stages
+constexpr int kStageArea = 24576;            // bytes of stages per CTA
 constexpr int kMaxStages = 6;
 
-template <typename T>
+// Three stages; six for int16 storage with one harmonic, the only variant that is the
+// faster for them with two CTAs per SM (2M int16 pixels of 414 dates: 1733 us with six, 1751
+// with three; with two harmonics 2045 and 2037, with three 2426 and 2319, on 8.4 Mi pixels 10.88
+// and 9.60 ms).
+//
+// kSolo: long histories leave one CTA per SM (the L2 budget below), so shared memory is
+// free.  With three harmonics and int16 storage it takes six stages, and the 21 basis
+// sums wait for the second solve in the ring, which is idle until pass B and is
+// lengthened for them.  1M pixels of 800 dates, history 640: 2.60 ms so, 2.75 with three stages and
+// the sums in registers; with two CTAs the sums in registers are the faster (400 dates: 1.09, 1.11 ms).
+template <int KH, typename T, bool kSolo>
 struct Stage {
     static constexpr int kBytes = kDates * kThreads * (int)sizeof(T);
-    static constexpr int kCount = kStageArea / kBytes;
+    static constexpr int kCount = sizeof(T) == 2 && (KH == 1 || kSolo) ? 6 : 3;
+    static_assert(kCount * kBytes <= kStageArea && kCount <= kMaxStages, "the stages fit their area");
 };
+constexpr int kStashed = Basis<3>::NBR;
+
 constexpr size_t kSmemMax = 112 * 1024;      // two CTAs per SM
 constexpr double kL2Budget = 80e6;           // bytes of history the resident pixels may hold in L2
 constexpr uint64_t kWaitNs = 2000000000ull;  // bound of every wait
 
 struct StreamParams {
-    int stages;        // stages in flight (int16)
     uint64_t wait_ns;  // bound of the consumers' stage waits (bfm_stage_wait_limit)
     const uint32_t* mask;
     int64_t m, mask_words;
@@ -120,12 +132,6 @@ __device__ __forceinline__ bool obs(int16_t raw, float& y) {
 struct Layout {
     size_t phi, xm, ring, stages, bars, total;
 };
-// With three harmonics and int16 storage the 21 basis sums wait for the second solve in the
-// ring, which is idle until pass B: in registers they make pass A' spill (500k pixels of 414
-// dates 654 us, 644 so with six stages fixed; float storage is the faster with its few spills, 9.24 ms against 9.34
-// on 8.4 Mi pixels).
-constexpr int kStashed = Basis<3>::NBR;
-
 __host__ __device__ inline size_t up128(size_t x) { return (x + 127) & ~(size_t)127; }
 
 __host__ __device__ inline Layout stream_layout(int N, int n, int K, int NB, int hmax) {
@@ -133,27 +139,26 @@ __host__ __device__ inline Layout stream_layout(int N, int n, int K, int NB, int
     L.phi = 0;
     L.xm = up128(sizeof(float) * (size_t)n * NB);
     L.ring = L.xm + up128(sizeof(float) * (size_t)(N - n) * K);
-    const int slots = K == 8 && hmax < kStashed ? kStashed : hmax;
-    L.stages = L.ring + up128(sizeof(float) * (size_t)slots * kThreads);
+    L.stages = L.ring + up128(sizeof(float) * (size_t)hmax * kThreads);
     L.bars = L.stages + (size_t)kStageArea;
-    // what decides whether a call takes this form: the ring alone, and 112 bytes
-    L.total = L.bars - up128(sizeof(float) * (size_t)slots * kThreads) + up128(sizeof(float) * (size_t)hmax * kThreads) +
-              2 * kMaxStages * sizeof(uint64_t) + 16;
+    // what decides whether a call takes this form; a launch takes 16 bytes more
+    // (kBarBytes; two CTAs of kSmemMax + 16 bytes fit an SM) and kSolo's ring
+    L.total = L.bars + 2 * kMaxStages * sizeof(uint64_t) + 16;
     return L;
 }
 
 // Barriers (with the one of the window starts), the abort flag and the window starts.
 constexpr size_t kBarBytes = 2 * kMaxStages * sizeof(uint64_t) + 32;
 
-template <int KH, typename T, bool kMask>
+template <int KH, typename T, bool kMask, bool kSolo>
 __global__ void __launch_bounds__(kThreads + 32, 2)
     stream_kernel(const __grid_constant__ CUtensorMap tmap, const StreamParams P) {
     using B = Basis<KH>;
     constexpr int K = B::K, NB = B::NB, NBR = B::NBR;
-    constexpr bool kStash = NBR == kStashed && sizeof(T) == 2;
     constexpr int G = kDates;                    // dates per stage
-    constexpr int kStageBytes = Stage<T>::kBytes;
-    const int kStages = sizeof(T) == 4 ? Stage<T>::kCount : P.stages;  // stages in flight
+    constexpr int kStageBytes = Stage<KH, T, kSolo>::kBytes;
+    constexpr int kStages = Stage<KH, T, kSolo>::kCount;  // stages in flight
+    static_assert(!kSolo || NBR == kStashed, "the ring holds the basis sums");
     extern __shared__ __align__(128) unsigned char smem[];
     const int n = P.n, N = P.N, hmax = P.hmax;
     const int64_t m = P.m;
@@ -357,27 +362,29 @@ __global__ void __launch_bounds__(kThreads + 32, 2)
             nonsingular = cholesky<K>(Gm, Lc, dinv);
             chol_solve<K>(Lc, dinv, Bv, b0);
         }
-        if constexpr (kStash) {
+        if constexpr (kSolo) {
 #pragma unroll
             for (int i = 0; i < NBR; ++i) ring[i * kThreads] = S[i];
         }
-
         const bool fit = np > K && nonsingular;
 
         // pass A': residuals r0 of the first solution, refinement sums c = X'M r0, and the
         // date of the window's oldest history observation (0-based valid rank n_p - h_p + 1).
         // rem: the valid history observations before that one; ~date once it is found (one
-        // register, which this pass has few of).
+        // register, which this pass has few of).  The valid dates of a batch are kept as
+        // bits and counted once: with a variant of the batch that looks date by date
+        // 2 Mi-pixel int16 calls of 414 dates took 2.22 ms, so 2.16 (K = 8).
         int rem = fit ? np - window() + 1 : np;
         float cr[K];
 #pragma unroll
         for (int a = 0; a < K; ++a) cr[a] = 0.f;
         float ss0 = 0.f;
-        auto passA2 = [&](int d0, auto full_c, auto scan_c, const T* st, uint32_t bits) {
+        auto passA2 = [&](int d0, auto full_c) {
             constexpr bool full = decltype(full_c)::value;
-            constexpr bool scan = decltype(scan_c)::value;  // a pixel of the warp may reach its window
             const int cnt = full ? G : n - d0;
-            const int left = rem >= 0 ? 1 : 0;
+            const T* st = acquire();
+            const uint32_t bits = mask_bits(d0, 0);
+            uint32_t vm = 0u;  // the valid dates
 #pragma unroll
             for (int u = 0; u < G; ++u) {
                 float y;
@@ -387,24 +394,21 @@ __global__ void __launch_bounds__(kThreads + 32, 2)
                 ss0 = fmaf(r, r, ss0);
 #pragma unroll
                 for (int a = 0; a < K; ++a) cr[a] = fmaf(ph[a], r, cr[a]);
-                if (scan)
-                    rem = v != 0.f && rem >= 0 ? (rem == 0 ? ~(d0 + u) : rem - 1) : rem;
-                else
-                    rem -= v != 0.f ? left : 0;
+                if (v != 0.f) vm |= 1u << u;
+            }
+            release();
+            const int valid = __popc(vm);
+            if ((unsigned)rem < (unsigned)valid) {  // the rem-th (from 0) of them
+#pragma unroll
+                for (int i = 0; i < G - 1; ++i) vm = i < rem ? vm & (vm - 1u) : vm;
+                rem = ~(d0 + __ffs((int)vm) - 1);
+            } else if (rem >= 0) {
+                rem -= valid;
             }
         };
         if (kMask) mb.open(0, lane);
-        for (d0 = 0; d0 < n && !bad; d0 += G) {
-            const T* st = acquire();
-            const uint32_t bits = mask_bits(d0, 0);
-            if (d0 + G > n)
-                passA2(d0, std::false_type{}, std::true_type{}, st, bits);
-            else if (__any_sync(~0u, (unsigned)rem < (unsigned)G))
-                passA2(d0, std::true_type{}, std::true_type{}, st, bits);
-            else
-                passA2(d0, std::true_type{}, std::false_type{}, st, bits);
-            release();
-        }
+        for (d0 = 0; d0 + G <= n && !bad; d0 += G) passA2(d0, std::true_type{});
+        if (d0 < n && !bad) passA2(d0, std::false_type{});
         const int wdate = rem < 0 ? ~rem : n;
         {
             const unsigned w = __reduce_min_sync(~0u, (unsigned)(active ? wdate : n));
@@ -415,7 +419,7 @@ __global__ void __launch_bounds__(kThreads + 32, 2)
         }
         float dl[K];
         {
-            if constexpr (kStash) {
+            if constexpr (kSolo) {
 #pragma unroll
                 for (int i = 0; i < NBR; ++i) S[i] = ring[i * kThreads];
             }
@@ -494,23 +498,33 @@ __global__ void __launch_bounds__(kThreads + 32, 2)
                 slot = take ? nslot : slot;
                 const float Wn = (W + r) - old;
                 W = take ? Wn : W;
-                Wu[u] = W;
-                amax = fmaxf(amax, fabsf(W));
-                blk += take ? W : 0.f;
+                Wu[u] = take ? Wn : 0.f;  // no window ends at an invalid date; 0 never crosses
+                amax = fmaxf(amax, fabsf(Wu[u]));
+                blk += Wu[u];
                 if (ext) {
                     wmax = take ? fmaxf(wmax, W) : wmax;
                     wmin = take ? fminf(wmin, W) : wmin;
                 }
                 Jf += v;
             }
-            // boundary test W^2 inv_scale^2 - b^2 > 0 (MO^2 > b^2).  The boundary grows with the
-            // position: a batch whose largest |MO| stays within it at its first position holds
-            // no crossing (lowered by 1e-5, more than its rounding, so that none is missed),
-            // and the dates are tested only in the others, until the first crossing.  Testing
-            // every date cost a logarithm and six more operations a date.
+            // boundary test W^2 inv_scale^2 - b^2 > 0 (MO^2 > b^2), until the first crossing and
+            // only in batches that may hold it.  Up to position e n_p the boundary is lambda,
+            // and the batch's largest |MO| decides.  Beyond, it grows with the position: a
+            // batch whose largest |MO| stays within it at its first position holds no crossing
+            // (lowered by 1e-5, more than its rounding, so that none is missed).  Testing every
+            // date cost a logarithm and six more operations a date; with one search for both
+            // parts, reading validity again and counting positions, calls in which
+            // many pixels cross got slower than that: 2 Mi int16 pixels of 200 dates, history 80,
+            // K = 8: 1.16 ms with every date tested, 1.21 with the one search, 1.05 so.
             if (brk < 0) {
                 auto bound = [&](float J) { return J > jlimf ? fmaf(lam2ln2, log2_fast(J), -blg) : P.lam2; };
-                if (fmaf(amax * amax, inv2, -(bound(J0) * 0.99999f)) > 0.f) {
+                if (Jf <= jlimf + 1.f) {  // the boundary is lambda all along
+                    if (fmaf(amax * amax, inv2, -P.lam2) > 0.f) {
+#pragma unroll
+                        for (int u = G - 1; u >= 0; --u)
+                            if (fmaf(Wu[u] * Wu[u], inv2, -P.lam2) > 0.f) brk = d0 + u;
+                    }
+                } else if (fmaf(amax * amax, inv2, -(bound(J0) * 0.99999f)) > 0.f) {
                     float J = J0;
 #pragma unroll
                     for (int u = 0; u < G; ++u) {
@@ -584,9 +598,9 @@ __global__ void __launch_bounds__(kThreads + 32, 2)
     }
 }
 
-template <int KH, typename T, bool kMask>
+template <int KH, typename T, bool kMask, bool kSolo>
 bfm_status launch_one(const CUtensorMap& tm, const StreamParams& P, int grid, size_t smem, cudaStream_t st) {
-    auto* fn = stream_kernel<KH, T, kMask>;
+    auto* fn = stream_kernel<KH, T, kMask, kSolo>;
     if (smem > 48 * 1024) {
         // the opt-in maximum, not this launch's size: launches of other sizes (other
         // scenes, other host threads) never find a smaller limit in place
@@ -599,14 +613,10 @@ bfm_status launch_one(const CUtensorMap& tm, const StreamParams& P, int grid, si
     return BFM_OK;
 }
 
-template <int KH>
-bfm_status launch_kh(const CUtensorMap& tm, const StreamParams& P, int dtype, int grid, size_t smem,
-                     cudaStream_t st) {
-    if (dtype == BFM_F32)
-        return P.mask ? launch_one<KH, float, true>(tm, P, grid, smem, st)
-                      : launch_one<KH, float, false>(tm, P, grid, smem, st);
-    return P.mask ? launch_one<KH, int16_t, true>(tm, P, grid, smem, st)
-                  : launch_one<KH, int16_t, false>(tm, P, grid, smem, st);
+template <int KH, typename T, bool kSolo = false>
+bfm_status launch_mask(const CUtensorMap& tm, const StreamParams& P, int grid, size_t smem, cudaStream_t st) {
+    return P.mask ? launch_one<KH, T, true, kSolo>(tm, P, grid, smem, st)
+                  : launch_one<KH, T, false, kSolo>(tm, P, grid, smem, st);
 }
 
 int stream_hmax(int n_hist, double h_frac) {
@@ -639,11 +649,6 @@ bfm_status launch_stream(const bfm_design_s* d, int dtype, const void* Y, const 
     }
     const size_t elt = dtype == BFM_F32 ? 4 : 2;
     StreamParams P{};
-    // int16 has room for six stages, but with rows of 16 MB the 96 dates that two CTAs then
-    // have in flight lie on more pages than the SM's address translations cover: 10.87 ms on
-    // 8.4 Mi pixels (K = 8), 9.77 with three.  At rows of 4 MB both take 2.36 ms on 2 Mi
-    // pixels, below that six are 1 % faster.
-    P.stages = (size_t)m * elt > ((size_t)4 << 20) ? 3 : Stage<int16_t>::kCount;
     P.wait_ns = stage_wait_ns();
     P.mask = mask;
     P.m = m;
@@ -682,10 +687,16 @@ bfm_status launch_stream(const bfm_design_s* d, int dtype, const void* Y, const 
     const int per_sm = 2.0 * kThreads * n_hist * (double)elt * sms <= kL2Budget ? 2 : 1;
     const int64_t ntiles = (m + kThreads - 1) / kThreads;
     const int grid = (int)(ntiles < (int64_t)per_sm * sms ? ntiles : (int64_t)per_sm * sms);
+    const bool f32 = elt == 4, solo = !f32 && d->k == 3 && per_sm == 1;
+    if (solo && P.hmax < kStashed) P.hmax = kStashed;
     const size_t smem = stream_layout(d->N, n_hist, d->K, basis_stride(d->k), P.hmax).bars + kBarBytes;
-    if (d->k == 1) return launch_kh<1>(tm, P, dtype, grid, smem, stream);
-    if (d->k == 2) return launch_kh<2>(tm, P, dtype, grid, smem, stream);
-    return launch_kh<3>(tm, P, dtype, grid, smem, stream);
+    if (d->k == 1)
+        return f32 ? launch_mask<1, float>(tm, P, grid, smem, stream) : launch_mask<1, int16_t>(tm, P, grid, smem, stream);
+    if (d->k == 2)
+        return f32 ? launch_mask<2, float>(tm, P, grid, smem, stream) : launch_mask<2, int16_t>(tm, P, grid, smem, stream);
+    return f32    ? launch_mask<3, float>(tm, P, grid, smem, stream)
+           : solo ? launch_mask<3, int16_t, true>(tm, P, grid, smem, stream)
+                  : launch_mask<3, int16_t>(tm, P, grid, smem, stream);
 }
 
 }  // namespace bfm
