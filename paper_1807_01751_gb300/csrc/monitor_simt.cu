@@ -126,7 +126,7 @@ __device__ __forceinline__ TileSmem tile_smem(unsigned char* smem_raw, const Mon
 // bar/bar_uses: the CTA's tile-load mbarrier and how often it has completed.
 // Returns with every warp done with shared memory except for a final
 // barrier the caller places before the next block.
-template <int KH, typename T, bool kMask>
+template <int KH, typename T, bool kMask, bool kPair = false>
 __device__ __forceinline__ void simt_block(const CUtensorMap* tmap, const MonitorParams& P, int64_t block,
                                            unsigned char* smem_raw, uint64_t* bar, uint32_t& bar_uses) {
     using B = Basis<KH>;
@@ -206,15 +206,15 @@ __device__ __forceinline__ void simt_block(const CUtensorMap* tmap, const Monito
 
     const SegParams sp{P.N, P.n_hist, P.h_frac, P.lambda, P.c_over_s, P.inv_s};
     Lane<KH> S;
-    phase1_gram<KH>(sp, w, obs, row, partf);
+    phase1_gram<KH, kPair>(sp, w, obs, row, partf);
     __syncthreads();
     phase2_solve<KH>(S, partf);
     __syncthreads();
-    phase3_refine<KH>(sp, w, S, obs, rowx, partf);
+    phase3_refine<KH, kPair>(sp, w, S, obs, rowx, partf);
     __syncthreads();
     phase4_sigma<KH>(sp, S, partf);
     __syncthreads();
-    phase5_resid<KH>(sp, w, S, obs, rowx, put_r, partf, putw);
+    phase5_resid<KH, kPair>(sp, w, S, obs, rowx, put_r, partf, putw);
     __syncthreads();
     phase6_offsets<KH>(w, S, partf);
     __syncthreads();  // phase 7 overwrites the segment totals phase 6 reads in every warp
@@ -243,9 +243,24 @@ __device__ __forceinline__ uint64_t* tile_bar(unsigned char* smem_raw, size_t sm
     return reinterpret_cast<uint64_t*>(smem_raw + smem_bytes - 16);
 }
 
+// The variants that carry their sums over dates in pairs (Sums): where that was measured to
+// be the faster; the others lose by it, up to 17 % (two harmonics, float, TMA: 400000 pixels of
+// 228 dates 548 us with pairs, 452 without).  Without TMA and mask: 100003 float pixels
+// of 500 dates, two harmonics, 422 us with, 433 without (one harmonic, int16: 580 and 532).  With
+// both: 24608 int16 pixels of 500 dates, three harmonics, 260 with, 277 without.  The
+// batch's kernel holds every variant and takes none.
+constexpr bool use_pairs(int kh, bool i16, bool tma, bool mask) {
+    return tma ? mask && (kh == 3 || (kh == 1 && i16)) : !mask && (kh == 2 || !i16);
+}
+
+// Resident CTAs asked of the compiler (0: none asked).  With three harmonics and int16 storage, staging
+// through registers and the pairs with a mask each go just past the 96 registers of
+// five CTAs per SM (100003 pixels of 120 dates, no TMA: 107 us with five, 121 with four).
+constexpr int min_ctas(int kh, bool i16, bool tma, bool mask) { return kh == 3 && i16 && tma == mask ? 5 : 0; }
+
 template <int KH, typename T, bool kTMA, bool kMask>
-__global__ void __launch_bounds__(kNW * 32) simt_kernel(const __grid_constant__ CUtensorMap tmap, const MonitorParams P,
-                                                       size_t smem_bytes) {
+__global__ void __launch_bounds__(kNW * 32, min_ctas(KH, sizeof(T) == 2, kTMA, kMask))
+    simt_kernel(const __grid_constant__ CUtensorMap tmap, const MonitorParams P, size_t smem_bytes) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     uint64_t* bar = tile_bar(smem_raw, smem_bytes);
     if (kTMA && threadIdx.x == 0) {
@@ -255,7 +270,8 @@ __global__ void __launch_bounds__(kNW * 32) simt_kernel(const __grid_constant__ 
     }
     __syncthreads();
     uint32_t uses = 0;
-    simt_block<KH, T, kMask>(kTMA ? &tmap : nullptr, P, blockIdx.x, smem_raw, bar, uses);
+    simt_block<KH, T, kMask, use_pairs(KH, sizeof(T) == 2, kTMA, kMask)>(kTMA ? &tmap : nullptr, P, blockIdx.x,
+                                                                         smem_raw, bar, uses);
 }
 
 // Persistent batched kernel: CTAs take 32-pixel blocks of any tile from a

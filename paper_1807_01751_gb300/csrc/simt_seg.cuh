@@ -146,9 +146,7 @@ __host__ __device__ __forceinline__ void chol_solve(const float (&L)[K][K], cons
 }
 
 // Two multiply-adds at once, c = a b + c by halves: one f32x2 instruction on the
-// device (each half rounds as fmaf does).  The sums over dates below carry their
-// accumulators in pairs of neighbouring basis functions: with
-// the tile staged by cp.async, 100003 float pixels of 228 dates in 186 us, before 211.
+// device (each half rounds as fmaf does).
 struct Pair {
     float x, y;
 };
@@ -164,12 +162,63 @@ __host__ __device__ __forceinline__ void fma_pair(Pair& c, float ax, float ay, f
 #endif
 }
 
+// Sums over dates of w q_i, i < n, each with its own accumulator or (kPair) in pairs of
+// neighbours.  Both give the same bits.  Which is the faster depends on what else
+// competes for registers and on how the tile arrives (monitor_simt.cu states the rule).
+template <int n, bool kPair>
+struct Sums {
+    float s[n];
+    __host__ __device__ __forceinline__ Sums() {
+#pragma unroll
+        for (int i = 0; i < n; ++i) s[i] = 0.f;
+    }
+    template <int m>
+    __host__ __device__ __forceinline__ void add(float w, const float (&q)[m]) {
+#pragma unroll
+        for (int i = 0; i < n; ++i) s[i] = fmaf(w, q[i], s[i]);
+    }
+    template <int m>
+    __host__ __device__ __forceinline__ void add1(float w, const float (&q)[m]) {  // q[0] = 1
+        s[0] += w;
+#pragma unroll
+        for (int i = 1; i < n; ++i) s[i] = fmaf(w, q[i], s[i]);
+    }
+    __host__ __device__ __forceinline__ float get(int i) const { return s[i]; }
+};
+template <int n>
+struct Sums<n, true> {
+    static constexpr int h = (n + 1) / 2;  // the last second half may be padding
+    Pair s[h];
+    __host__ __device__ __forceinline__ Sums() {
+#pragma unroll
+        for (int i = 0; i < h; ++i) s[i] = Pair{0.f, 0.f};
+    }
+    template <int m>
+    __host__ __device__ __forceinline__ void add(float w, const float (&q)[m]) {
+        static_assert(2 * h <= m, "a value for the padding");
+#pragma unroll
+        for (int i = 0; i < h; ++i) fma_pair(s[i], w, w, q[2 * i], q[2 * i + 1]);
+    }
+    template <int m>
+    __host__ __device__ __forceinline__ void add1(float w, const float (&q)[m]) {
+        add(w, q);
+    }
+    __host__ __device__ __forceinline__ float get(int i) const { return i & 1 ? s[i / 2].y : s[i / 2].x; }
+};
+
 // x_t . beta as two interleaved chains
-template <int K>
+template <int K, bool kPair>
 __host__ __device__ __forceinline__ float dot_x(const float (&x)[K], const float (&beta)[K]) {
     Pair f{0.f, 0.f};
 #pragma unroll
-    for (int i = 0; i < K; i += 2) fma_pair(f, x[i], x[i + 1], beta[i], beta[i + 1]);
+    for (int i = 0; i < K; i += 2) {
+        if constexpr (kPair) {
+            fma_pair(f, x[i], x[i + 1], beta[i], beta[i + 1]);
+        } else {
+            f.x = fmaf(x[i], beta[i], f.x);
+            f.y = fmaf(x[i + 1], beta[i + 1], f.y);
+        }
+    }
     return f.x + f.y;
 }
 
@@ -221,18 +270,14 @@ struct Lane {
 // PART(w, i) -> float& : partial slot i of warp w for this lane.
 
 // ---- phase 1: masked basis sums over this warp's history segment -------------------
-template <int KH, class Obs, class Row, class Part>
+template <int KH, bool kPair, class Obs, class Row, class Part>
 __host__ __device__ __forceinline__ void phase1_gram(const SegParams& P, int w, Obs obs, Row row, Part part) {
     using B = Basis<KH>;
     constexpr int K = B::K, NB = B::NB, NBR = B::NBR;
     int s0, s1;
     segment(P.n_hist, w, s0, s1);
-    constexpr int NP = (NBR + 1) / 2;  // NBR is odd: the last pair's second half is padding
-    Pair a[NP], bb[K / 2];
-#pragma unroll
-    for (int i = 0; i < NP; ++i) a[i] = Pair{0.f, 0.f};
-#pragma unroll
-    for (int i = 0; i < K / 2; ++i) bb[i] = Pair{0.f, 0.f};
+    Sums<NBR, kPair> a;
+    Sums<K, kPair> bb;
     float ymax = 0.f;
 #pragma unroll 2
     for (int t = s0; t < s1; ++t) {
@@ -242,15 +287,13 @@ __host__ __device__ __forceinline__ void phase1_gram(const SegParams& P, int w, 
         ymax = fmaxf(ymax, fabsf(yw));
         float q[NB];
         row(t, q);
-#pragma unroll
-        for (int l = 0; l < NP; ++l) fma_pair(a[l], wt, wt, q[2 * l], q[2 * l + 1]);  // q[0] = 1
-#pragma unroll
-        for (int i = 0; i < K / 2; ++i) fma_pair(bb[i], yw, yw, q[2 * i], q[2 * i + 1]);
+        a.add1(wt, q);
+        bb.add1(yw, q);
     }
 #pragma unroll
-    for (int i = 0; i < NBR; ++i) part(w, i) = i & 1 ? a[i / 2].y : a[i / 2].x;
+    for (int i = 0; i < NBR; ++i) part(w, i) = a.get(i);
 #pragma unroll
-    for (int i = 0; i < K; ++i) part(w, NBR + i) = i & 1 ? bb[i / 2].y : bb[i / 2].x;
+    for (int i = 0; i < K; ++i) part(w, NBR + i) = bb.get(i);
     part(w, NBR + K) = ymax;
 }
 
@@ -282,15 +325,13 @@ __host__ __device__ __forceinline__ void phase2_solve(Lane<KH>& S, Part part) {
 }
 
 // ---- phase 3: refinement sums over this warp's history segment ------------------
-template <int KH, class Obs, class RowX, class Part>
+template <int KH, bool kPair, class Obs, class RowX, class Part>
 __host__ __device__ __forceinline__ void phase3_refine(const SegParams& P, int w, const Lane<KH>& S, Obs obs,
                                                        RowX rowx, Part part) {
     constexpr int K = Basis<KH>::K;
     int s0, s1;
     segment(P.n_hist, w, s0, s1);
-    Pair cc[K / 2];
-#pragma unroll
-    for (int i = 0; i < K / 2; ++i) cc[i] = Pair{0.f, 0.f};
+    Sums<K, kPair> cc;
     float ss = 0.f;
 #pragma unroll 2
     for (int t = s0; t < s1; ++t) {
@@ -298,13 +339,12 @@ __host__ __device__ __forceinline__ void phase3_refine(const SegParams& P, int w
         const bool v = obs(t, y);
         float x[K];
         rowx(t, x);
-        const float r = v ? (y - dot_x<K>(x, S.beta)) : 0.f;
+        const float r = v ? (y - dot_x<K, kPair>(x, S.beta)) : 0.f;
         ss = fmaf(r, r, ss);
-#pragma unroll
-        for (int i = 0; i < K / 2; ++i) fma_pair(cc[i], r, r, x[2 * i], x[2 * i + 1]);
+        cc.add(r, x);
     }
 #pragma unroll
-    for (int i = 0; i < K; ++i) part(w, i) = i & 1 ? cc[i / 2].y : cc[i / 2].x;
+    for (int i = 0; i < K; ++i) part(w, i) = cc.get(i);
     part(w, K) = ss;
 }
 
@@ -346,7 +386,7 @@ __host__ __device__ __forceinline__ void phase4_sigma(const SegParams& P, Lane<K
 // ---- phase 5: residuals, segment-local compacted prefix sums ------------------------
 // put_s(slot, v) writes slot (always <= the date being read, inside the
 // segment); putw(w, i, bits) stores validity word i of this warp's segment.
-template <int KH, class Obs, class RowX, class PutS, class Part, class PutW>
+template <int KH, bool kPair, class Obs, class RowX, class PutS, class Part, class PutW>
 __host__ __device__ __forceinline__ void phase5_resid(const SegParams& P, int w, const Lane<KH>& S, Obs obs,
                                                       RowX rowx, PutS put_s, Part part, PutW putw) {
     constexpr int K = Basis<KH>::K;
@@ -361,7 +401,7 @@ __host__ __device__ __forceinline__ void phase5_resid(const SegParams& P, int w,
         const bool v = obs(t, y);
         float x[K];
         rowx(t, x);
-        const float r = y - dot_x<K>(x, S.beta);
+        const float r = y - dot_x<K, kPair>(x, S.beta);
         if (v) {
             comp_add(sh, sl, r);
             put_s(s0 + jl, sh + sl);
