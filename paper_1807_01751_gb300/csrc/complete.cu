@@ -1128,10 +1128,16 @@ bfm_status launch_complete(bfm_design_s* d, int dtype, const void* Y, const uint
     if (staged && !P.mask && shared == BFM_PX_OK) {
         // pixel pairs: scenes of at least a tile of 512 pixels per SM (smaller ones leave SMs to
         // the other kernel's two CTAs of 256) whose tables, ring and three stages fit, with
-        // the history of the resident pixels within the L2 budget
+        // the history of the resident pixels within the L2 budget.  Int16 scenes of a few tiles
+        // more than SMs stay with the other kernel, whose second round is of tiles half the
+        // size, with the map of the largest |MO| and three harmonics up to half as
+        // many more (77832 pixels of 414 dates: 88.6 us against 91.9 here, 92.6 with the map;
+        // 100000: 95.0 against 94.8 and 96.5; 120000: 116 against 97 and 99).  Float is the
+        // faster here throughout (77832: 94.7 against 90.0).
         const PairLayout pl = pair_layout(d->N, n_hist, d->K, P.h);
-        const int64_t ptiles = (m + kPairPx - 1) / kPairPx;
-        if (pl.nstages && ptiles >= (int64_t)sms && (double)kPairPx * n_hist * (double)elt * sms <= kL2Budget) {
+        const int64_t ptiles = (m + kPairPx - 1) / kPairPx, rest = ptiles - sms;
+        const int64_t few = elt == 4 ? 0 : !maxmo ? sms / 32 : d->k == 3 ? sms / 2 : sms / 16;
+        if (pl.nstages && (rest == 0 || rest > few) && (double)kPairPx * n_hist * (double)elt * sms <= kL2Budget) {
             const int pgrid = (int)(ptiles < sms ? ptiles : sms);
             if (dtype == BFM_F32)
                 return d->k == 1   ? launch_pair<1, float>(tm, P, pgrid, pl.total, stream)
