@@ -45,6 +45,13 @@ constexpr int kPer = 2;                               // consecutive steps of a 
 constexpr int kSteps = 32 * kPer;                     // steps of a warp at a time
 constexpr double kE = 2.718281828459045235360287;
 constexpr size_t kMaxRingBytes = 200 * 1024;          // rings of a block
+// Up to here two blocks share an SM (228 KB, 4 KB of each for the tables and the system).
+// Beyond, four warps an SM wait on one another's draws, and drawing the lagged steps again at
+// full occupancy is the faster: 20000 paths, h = 1, T = 1.8, ring against second draw: G = 2000
+// 1.67 and 2.07 ms, 3000 2.77 and 2.96, 4000 5.51 and 3.84, 6000 8.12 and 5.61.  With no
+// more paths than one block per SM takes, the ring stays ahead (200 paths, G = 6000:
+// 457 and 578 us).
+constexpr size_t kTwoRingBytes = 110 * 1024;
 
 struct LambdaParams {
     int G, nsteps, ih, reps;
@@ -122,8 +129,8 @@ __global__ void __launch_bounds__(kSelThreads) kth_smallest(double* v, int n, in
     if (threadIdx.x == 0) v[n] = __longlong_as_double((long long)prefix);
 }
 
-// One path per warp.  kRing: W(t - h) from the ring; otherwise (h G too long for
-// shared memory) rebuilt from the stream by a second draw of the lagged steps.
+// One path per warp.  kRing: W(t - h) from the ring; otherwise (h G too long for two
+// blocks per SM) rebuilt from the stream by a second draw of the lagged steps.
 template <bool kRing>
 __global__ void __launch_bounds__(32 * kWarps)
     lambda_paths(const __grid_constant__ fixedpt::LogTable tab, const LambdaParams P) {
@@ -222,12 +229,10 @@ const fixedpt::LogTable& log_table() {
 }
 
 template <bool kRing>
-cudaError_t launch_paths(const LambdaParams& P, size_t smem, cudaStream_t st) {
+cudaError_t launch_paths(const LambdaParams& P, size_t smem, int sms, cudaStream_t st) {
     auto* fn = lambda_paths<kRing>;
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxRingBytes);
-    int dev = 0, sms = 0, per = 0;
-    if (e == cudaSuccess) e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    int per = 0;
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, 32 * kWarps, smem);
     if (e != cudaSuccess) return e;
     const int64_t want = ((int64_t)P.reps + kWarps - 1) / kWarps, most = (int64_t)sms * (per < 1 ? 1 : per);
@@ -273,9 +278,16 @@ extern "C" bfm_status bfm_lambda(double alpha, double h, double T, int G, int re
     P.h = h < 1.0 ? (uint64_t)std::ldexp(h, 64) : 0ull;
     P.stats = d_stats;
     const int64_t slots = ((int64_t)ih + 2 * kSteps - 1) / kSteps * kSteps;
-    const bool ring = (size_t)slots * kWarps * 8 <= kMaxRingBytes;
+    int dev = 0, sms = 0;
+    e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) {
+        cudaFreeAsync(d_stats, st);
+        return cuda_fail(e, "bfm_lambda: device attributes");
+    }
+    const bool ring = (size_t)slots * kWarps * 8 <= (reps <= kWarps * sms ? kMaxRingBytes : kTwoRingBytes);
     P.ring = ring ? (int)slots : 0;
-    e = ring ? launch_paths<true>(P, (size_t)slots * kWarps * 8, st) : launch_paths<false>(P, 0, st);
+    e = ring ? launch_paths<true>(P, (size_t)slots * kWarps * 8, sms, st) : launch_paths<false>(P, 0, sms, st);
     // (1 - alpha) empirical quantile: the ceil((1 - alpha) reps)-th smallest
     long q = (long)std::ceil((1.0 - alpha) * (double)reps) - 1;
     q = q < 0 ? 0 : (q >= reps ? reps - 1 : q);
