@@ -21,6 +21,8 @@ A, B, M = 0xA0761D6478BD642F, 0xE7037ED1A0B428DB, 1 << 64
     (1.0, 1.1, 3360, 9000),   # the longest ring with two blocks per SM
     (1.0, 1.1, 3600, 20000),  # the lagged steps drawn again, several rounds
     (1.0, 1.1, 3600, 300),    # a ring with one block per SM
+    (1.0, 1.2, 1, 5000),      # all statistics 0: the quantile among equal values
+    (0.5, 2.0, 2, 3000),
 ])
 def test_rounds(h, T, G, reps):
     if not torch.cuda.is_available():
