@@ -511,11 +511,12 @@ __global__ void __launch_bounds__(kThreads + 32, 2)
             // only in batches that may hold it.  Up to position e n_p the boundary is lambda,
             // and the batch's largest |MO| decides.  Beyond, it grows with the position: a
             // batch whose largest |MO| stays within it at its first position holds no crossing
-            // (lowered by 1e-5, more than its rounding, so that none is missed).  Testing every
-            // date cost a logarithm and six more operations a date; with one search for both
-            // parts, reading validity again and counting positions, calls in which
-            // many pixels cross got slower than that: 2 Mi int16 pixels of 200 dates, history 80,
-            // K = 8: 1.16 ms with every date tested, 1.21 with the one search, 1.05 so.
+            // (lowered by 1e-5, more than its rounding, so that none is missed), and the search
+            // counts positions, without branches.  Testing every date cost a logarithm and six
+            // more operations a date; with one branching search for both parts, calls in which
+            // many pixels cross got slower than that.  Int16, K = 8: 2 Mi pixels of 200 dates,
+            // history 80: 1.16 ms with every date tested, 1.21 with the one search, 1.05 so;
+            // 370600 pixels of 168 dates, history 37: 183, 208 and 156 us.
             if (brk < 0) {
                 auto bound = [&](float J) { return J > jlimf ? fmaf(lam2ln2, log2_fast(J), -blg) : P.lam2; };
                 if (Jf <= jlimf + 1.f) {  // the boundary is lambda all along
@@ -529,10 +530,9 @@ __global__ void __launch_bounds__(kThreads + 32, 2)
 #pragma unroll
                     for (int u = 0; u < G; ++u) {
                         float y;
-                        if (get(st, bits, u, cnt, full, y) != 0.f) {
-                            if (brk < 0 && fmaf(Wu[u] * Wu[u], inv2, -bound(J)) > 0.f) brk = d0 + u;
-                            J += 1.f;
-                        }
+                        const bool over = fmaf(Wu[u] * Wu[u], inv2, -bound(J)) > 0.f;
+                        brk = brk < 0 && over ? d0 + u : brk;
+                        J += get(st, bits, u, cnt, full, y);
                     }
                 }
             }
