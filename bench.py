@@ -42,9 +42,9 @@ sys.path.insert(0, ROOT)
 METRIC = "BFAST-monitor pixels/s at 8.4M px x 414 dates; p50/p99 tile latency"
 # DRAM bytes per pixel per launch from the ncu captures summarised in
 # profiles/ (None once the kernel changes after the capture).
-TRAFFIC_PER_PX = {"f32": (1.78515e9 / 1048576,), "f32simt": (1.78385e9 / 1048576,), "f32stream": (1.86174e9 / 1048576,),
+TRAFFIC_PER_PX = {"f32": (1.78515e9 / 1048576,), "f32simt": (1.78523e9 / 1048576,), "f32stream": (1.86088e9 / 1048576,),
                   "i16": (0.911513e9 / 1048576,), "f32hybrid": (1.83945e9 / 1048576,), "i16hybrid": (0.914645e9 / 1048576,),
-                  "i16stream": (0.912723e9 / 1048576,), "f32complete": (1.82763e9 / 1048576,)}
+                  "i16stream": (0.912998e9 / 1048576,), "f32complete": (1.82763e9 / 1048576,)}
 SAMPLE_PX = 4096  # pixels of each timed form checked against the oracle (outside the timed region)
 
 WORKLOAD = "c2: full scene 8,388,608 px x 414 dates, n_hist=228, K=8, f=23, h=0.25, plain float32"
@@ -336,9 +336,8 @@ def run_tiles_and_serving(bfm, synth, torch, dev, stream):
 
     c4["batched_launch"] = dict(batched(bfm.BFM_ALGO_AUTO),
                                 form="one CUDA-graph replay: persistent hybrid kernels per (k, storage, layout) "
-                                     "group, persistent tensor-core kernels per (k, storage, CTAs per SM) group for "
-                                     "the tiles whose ring does not fit the hybrid form, the CUDA-core kernel for "
-                                     "the rest")
+                                     "group, one tensor-core kernel node for each tile "
+                                     "whose ring does not fit the hybrid form, the CUDA-core kernel for the rest")
     c4["batched_launch_tensor_core_forms"] = dict(batched(bfm.BFM_ALGO_MMA),
                                                   form="the same batch limited to the tensor-core and CUDA-core forms")
 

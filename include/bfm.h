@@ -225,8 +225,9 @@ bfm_status bfm_monitor_ext(bfm_design_t d, const void *Y, int dtype, const uint3
  * with h rounded to whole steps.  *lambda_out receives the
  * ceil((1 - alpha) * reps)-th smallest statistic; stats_host (nullable,
  * host, reps doubles) receives all of them.  Runs on `stream` and returns
- * when done (synchronising it).  The paths are 64-bit fixed-point words whose
- * step is finer than the rounding of a double; the results are doubles.
+ * when done (synchronising it).  The paths are 64-bit fixed-point words of
+ * absolute step 2^(ceil(log2(40 sqrt T)) - 62) (2^-56 at T = 1.8); the
+ * statistics are doubles and agree with FP64 simulations to about 1e-14.
  * Errors: BFM_EINVAL (0 < alpha < 1, 0 < h <= 1, T > 1, G >= 1, reps >= 1
  * and round(h * G) >= 1 are required), BFM_ECUDA.
  */

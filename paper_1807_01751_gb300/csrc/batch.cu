@@ -10,8 +10,8 @@
 // the kernel a single call launches over the tile's own 128-pixel blocks.  The
 // CUDA-core tiles go to one persistent kernel whose CTAs take 32-pixel blocks
 // from a device counter, `grab` at a time.  The counter reset (one memset
-// node), the hybrid kernels (a chain after it) and, after them in parallel
-// branches, the tensor-core tile nodes and the CUDA-core kernel form one
+// node), the hybrid kernels (parallel branches after it) and, after all of
+// them in parallel branches, the tensor-core tile nodes and the CUDA-core kernel form one
 // graph, instantiated once and replayed.  An autotuner times (CTAs per SM,
 // grab) for the CUDA-core kernel on the batch itself and caches the best pair
 // per batch signature.

@@ -503,7 +503,7 @@ __global__ void __launch_bounds__(kStaged ? kThreads + 32 : kThreads, 2)
 // read as they are: in pass 1 neighbouring coefficients of one pixel (M' row x y), in
 // the residuals two dates of one pixel (the regressors are stored by date pairs), in the
 // window sums the two pixels.  (Tables holding each value twice, pixels paired
-// throughout, kept the shared-memory pipe 71 % busy: 4.93 ms.)
+// throughout, kept the shared-memory pipe 71 % busy: 4.75 ms.)
 // A CTA per SM owns 512 pixels.  8.4 Mi float pixels of 414 dates: 5.55 -> 4.36 ms, now
 // with two warps a scheduler issuing on 52 % of its cycles.
 

@@ -17,8 +17,9 @@
 // What bounds it: the normals.  In FP64 (one thread per path, the lagged
 // W(t - h) rebuilt by a second pass over the stream) 1e5 paths of 1816 steps
 // took 52.6 ms, nearly all of it FP64 issue.  Here the normals come from
-// lambda_fixed.cuh (integer arithmetic) and W is a 64-bit fixed-point word, whose
-// step 2^-frac is finer than the rounding of an FP64 W: against 113-bit arithmetic,
+// lambda_fixed.cuh (integer arithmetic) and W is a 64-bit fixed-point word with steps of
+// 2^-frac (2^-56 at T = 1.8; a double is finer only for |W| below a sixteenth), which
+// sums without further rounding: against 113-bit arithmetic,
 // over 150 such paths, the statistic is off by 7.2e-17 on average and 2.2e-16 at
 // most; in FP64 by 6.6e-16 and 4.8e-15.  Fixed-point sums do not
 // depend on their order, so a warp takes one path, 64 steps at a time: every lane

@@ -886,9 +886,11 @@ constexpr size_t kSmemTwo = 115712;  // shared memory per CTA with two CTAs on a
 // (only with more than 16 basis sums), two A buffers, the valid bytes and the pair
 // exchange floats, later the MOSUM ring; the Y stages; barriers.  Y has 3 (float)
 // or 6 (int16) stages, or as few as 2 (float) or 4 (int16) where that lets two CTAs
-// share an SM.  On 1.95 Mi int16 pixels of 586 dates (history 347, ring of 103 slots, 116 KB
-// with six stages and 112 with five) two CTAs took 5.03 ms, one 8.50; with the chunk and
-// group hand-offs per warp and ring and stage slots counted along, 4.49.
+// share an SM (in both types 1.71 to 1.73 times as fast: 1M pixels of 600 dates, history
+// 360: float 3.99 ms with three stages, 2.32 with two; int16 4.08 with six, 2.38 with four).
+// On 1.95 Mi int16 pixels of 586 dates (history 347, ring of 103 slots, 116 KB with six
+// stages and 112 with five) two CTAs took 5.03 ms, one 8.50; with the chunk and group
+// hand-offs per warp and ring and stage slots counted along, 4.49.
 MmaLayout mma_layout(int npad, int nhpad, int k, int ring, int elt) {
     MmaLayout L{};
     const size_t ta = (size_t)(npad / 8) * kTabLbo;

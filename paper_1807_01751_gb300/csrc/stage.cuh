@@ -53,7 +53,7 @@ __device__ __forceinline__ void tma_box(void* dst, const CUtensorMap* map, uint6
 // lane p with pixel p's bit of date d + u in bit u.  The words of the next 32
 // dates are loaded one step ahead.  Against one word load per date and pixel,
 // each exposed in the per-date chain, a 1 Mi-pixel float call of 414 dates of the
-// hybrid form went from 3.26 to 1.45 ms (1.10 with its two groups).  Warp-collective.
+// hybrid form went from 3.26 to 1.45 ms (1.13 with its two groups).  Warp-collective.
 struct MaskBits {
     const uint32_t* col;  // the warp's word column
     size_t ws;            // words per date

@@ -5,8 +5,9 @@
 // (pass A, A', B over the history, pass C over the monitoring dates), in
 // stages filled by 2-D TMA boxes (256 pixels x 8 dates) that a producer
 // warp issues up to a full ring ahead; the history stays in L2 between its
-// passes (evict-last hints, a grid sized to the L2), so Y is read once from DRAM.  Per pixel (Section 2.1, Eq. 3-6, Algorithm 1 with
-// missing values masked, as in the other forms):
+// passes (evict-last hints, a grid sized to the L2), so Y is read once from
+// DRAM.  Per pixel (Section 2.1, Eq. 3-6, Algorithm 1 with missing values
+// masked, as in the other forms):
 //   A   masked sums of the basis functions of bfm::Basis over the valid
 //       history dates -> Gram matrix G (identities of gram_from_sums) and
 //       X'My; valid count n_p; max |y|.  Cholesky of G with the rank test of
@@ -691,9 +692,11 @@ bfm_status launch_stream(const bfm_design_s* d, int dtype, const void* Y, const 
     if (solo && P.hmax < kStashed) P.hmax = kStashed;
     const size_t smem = stream_layout(d->N, n_hist, d->K, basis_stride(d->k), P.hmax).bars + kBarBytes;
     if (d->k == 1)
-        return f32 ? launch_mask<1, float>(tm, P, grid, smem, stream) : launch_mask<1, int16_t>(tm, P, grid, smem, stream);
+        return f32 ? launch_mask<1, float>(tm, P, grid, smem, stream)
+                   : launch_mask<1, int16_t>(tm, P, grid, smem, stream);
     if (d->k == 2)
-        return f32 ? launch_mask<2, float>(tm, P, grid, smem, stream) : launch_mask<2, int16_t>(tm, P, grid, smem, stream);
+        return f32 ? launch_mask<2, float>(tm, P, grid, smem, stream)
+                   : launch_mask<2, int16_t>(tm, P, grid, smem, stream);
     return f32    ? launch_mask<3, float>(tm, P, grid, smem, stream)
            : solo ? launch_mask<3, int16_t, true>(tm, P, grid, smem, stream)
                   : launch_mask<3, int16_t>(tm, P, grid, smem, stream);
